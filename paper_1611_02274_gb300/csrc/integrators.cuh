@@ -105,7 +105,7 @@ struct RkckF64 {
     using TM = Team<W>;
     typename Model::template Sys<double> sys;
     double y[P], k1[P], k2[P], k3[P], k4[P], k5[P];
-    double t, tend, h, hmax, delta, rtol;
+    double t, tend, h, hmax, delta, rtol, rrtol;
     int32_t n_acc, n_rej, status, max_att, stage;
 
     __device__ void init(const BatchArgs& a, const typename Model::Ctx& ctx, const TM& tm, int64_t i) {
@@ -118,6 +118,7 @@ struct RkckF64 {
         t = a.t0_of(i);
         tend = a.tend_of(i);
         rtol = a.rtol_of(i);
+        rrtol = xm::reciprocal(rtol);
         hmax = fabs(tend - t);
         h = 0.5 * fabs(tend - t);
         if (carry_warm(a, i) && a.carry[a.cidx(i, kCarryH)] > 0.0) h = a.carry[a.cidx(i, kCarryH)];
@@ -131,12 +132,13 @@ struct RkckF64 {
     // top of the rkckDriver loop: finished?  attempt cap, then clamp h
     __device__ void loop_top() {
         stage = 0;
-        if (!(t < tend)) return;
+        const double left = tend - t;  // positive exactly when t < tend
+        if (!xm::is_pos(left)) return;
         if (n_acc + n_rej >= max_att) {
             status = ODE_ST_MAX_ATTEMPTS;
             return;
         }
-        h = fmin(tend - t, h);
+        h = xm::min_nn(left, h);
         stage = 1;
     }
 
@@ -220,18 +222,24 @@ struct RkckF64 {
             yt[s] = y[s] + ck::C1 * k1[s] + ck::C3 * k3[s] + ck::C4 * k4[s] + ck::C6 * k6;
             const double ye = ck::DC1 * k1[s] + ck::DC3 * k3[s] + ck::DC4 * k4[s] + ck::DC5 * k5[s] + ck::DC6 * k6;
             if (sys.comp(tm, s) >= 0) {
-                if (isnan(ye)) nan_flag = true;
-                err = fmax(err, fabs(ye) / (fabs(y[s]) + fabs(k1[s]) + delta));
+                if (xm::is_nan(ye)) nan_flag = true;
+                err = xm::max_nn(err, fabs(ye) / (fabs(y[s]) + fabs(k1[s]) + delta));
             }
         }
-        err = tm.max(err) / rtol;
-        nan_flag = tm.any(nan_flag);
-        if (err > 1.0 || isnan(err) || nan_flag) {
+        if constexpr (W > 1) {
+#pragma unroll
+            for (int o = W / 2; o > 0; o >>= 1) err = xm::max_nn(err, shfl_xor(tm.mask, err, o, W));
+        }
+        err = xm::div_by(err, rtol, rrtol);
+        nan_flag = tm.any(nan_flag) || xm::is_nan(err);
+        const bool reject = nan_flag || xm::lt_nn(1.0, err);
+        const double fac = xm::pow_series(err, reject ? kPshrnk : kPgrow);
+        if (reject) {
             n_rej += 1;
-            if (isnan(err) || nan_flag)
+            if (nan_flag)
                 h = h * kP1;
             else
-                h = fmax(kSafety * h * xm::pow_series(err, kPshrnk), kP1 * h);
+                h = xm::max_nn(kSafety * h * fac, kP1 * h);
             if (h < 1.0e-20 || t + h == t) {
                 status = ODE_ST_H_UNDERFLOW;
                 stage = 0;
@@ -242,16 +250,16 @@ struct RkckF64 {
         }
         n_acc += 1;
         t = t + h;
-        if (err > kErrcon)
-            h = kSafety * h * xm::pow_series(err, kPgrow);
+        if (xm::lt_nn(kErrcon, err))
+            h = kSafety * h * fac;
         else
             h = h * 5.0;
-        h = fmax(1.0e-20, fmin(hmax, h));
+        h = xm::max_nn(1.0e-20, xm::min_nn(hmax, h));
         bool bad = false;
 #pragma unroll(P <= 64 ? P : 4)
         for (int s = 0; s < P; ++s) {
             y[s] = yt[s];
-            if (sys.comp(tm, s) >= 0 && !isfinite(yt[s])) bad = true;
+            if (sys.comp(tm, s) >= 0 && !xm::is_finite(yt[s])) bad = true;
         }
         if (tm.any(bad)) {
             status = ODE_ST_NONFINITE;
@@ -295,6 +303,7 @@ struct RkcF64 {
     typename Model::template Sys<double> sys;
     double yn[P], Fn[P], v[P], w1[P], w2[P];  // w1 = w_{j-1}, w2 = w_{j-2}
     double t, tend, rtol, atol, hmax, hmin, h, h_old, err_old, sigma;
+    double lerr_old, rn;                        // log err_old; 1 / n (xm::div_by)
     double dynrm, sig;                          // power method in progress
     StageCoef cur;                              // coefficients of the current stage
     CoefSource cs;
@@ -307,6 +316,8 @@ struct RkcF64 {
     __device__ void init(const BatchArgs& a, const typename Model::Ctx& ctx, const TM& tm, int64_t i) {
         sys.load(ctx, tm, a.params[i], a.neq_of(i));
         n = a.neq_of(i);
+        rn = xm::reciprocal((double)n);
+        lerr_old = 0.0;
         idx = i;
         n_est = 0;
 #pragma unroll(P <= 64 ? P : 4)
@@ -335,6 +346,7 @@ struct RkcF64 {
             sigma = a.carry[a.cidx(i, kCarrySigma)];
             h_old = a.carry[a.cidx(i, kCarryHold)];
             err_old = a.carry[a.cidx(i, kCarryErrOld)];
+            lerr_old = xm::log_series(err_old);
             num_step = (int)a.carry[a.cidx(i, kCarryNumStep)];
             sr_step = (int)a.carry[a.cidx(i, kCarrySrStep)];
             rejected = (int)a.carry[a.cidx(i, kCarryRejected)] != 0;
@@ -412,7 +424,8 @@ struct RkcF64 {
 
     // top of the rkcDriver loop
     __device__ void loop_top(const BatchArgs& a, const TM& tm) {
-        if (!(t < tend)) {
+        const double left = tend - t;  // positive exactly when t < tend
+        if (!xm::is_pos(left)) {
             phase = PH_DONE;
             return;
         }
@@ -421,7 +434,7 @@ struct RkcF64 {
             phase = PH_DONE;
             return;
         }
-        if (1.1 * h >= fabs(tend - t)) h = fabs(tend - t);
+        if (xm::le_nn(left, 1.1 * h)) h = left;
         if (!have_sigma || rejected || (num_step % kSpecradEvery == 0 && sr_step != num_step)) {
             if (a.specrad == ODE_SPECRAD_GERSHGORIN) {  // the bound replaces the power method
                 sigma = sys.gershgorin(tm, yn);
@@ -523,7 +536,7 @@ struct RkcF64 {
     }
 
     __device__ void after_sr(const BatchArgs& a) {
-        if (h < kUround) {
+        if (xm::lt_nn(h, kUround)) {
             // initial step: trial Euler step of size 1/sigma
             h = hmax;
             if (sigma * h > 1.0) h = 1.0 / sigma;
@@ -550,9 +563,19 @@ struct RkcF64 {
         stage_begin(a);
     }
 
+    // (int)sqrt(v): the FP32 root decides it unless it lies within its own
+    // rounding of an integer (two roundings, below 2^-22 relative)
+    __device__ static int floor_sqrt(double v) {
+        const float s = sqrtf((float)v);
+        const int k = (int)s;
+        const float frac = s - (float)k, slack = s * 4.0e-7f;
+        if (s < 1.0e6f && frac > slack && frac < 1.0f - slack) return k;
+        return (int)sqrt(v);
+    }
+
     // stage count, then w_0 = y_n, w_1 = w_0 + mu~_1 h F_n (Eqs. E:rkc0, E:rkc1)
     __device__ void stage_begin(const BatchArgs& a) {
-        m = 1 + (int)sqrt(1.54 * h * sigma + 1.0);
+        m = 1 + floor_sqrt(1.54 * h * sigma + 1.0);
         if (m > mmax) {
             m = mmax;
             h = (double)(m * m - 1) / (1.54 * sigma);
@@ -591,19 +614,20 @@ struct RkcF64 {
 #pragma unroll(P <= 64 ? P : 4)
         for (int s = 0; s < P; ++s) {
             double e = 0.8 * (yn[s] - w1[s]) + 0.4 * h * (Fn[s] + f[s]);
-            e = e / (atol + rtol * fmax(fabs(w1[s]), fabs(yn[s])));
+            e = e / (atol + rtol * xm::max_mag(w1[s], yn[s]));
             sq[s] = e * e;
         }
-        const double err = sqrt(sys.ordered_sum(tm, sq) / (double)n);
-        if (isnan(err)) {
+        const double err = sqrt(xm::div_by(sys.ordered_sum(tm, sq), xm::small_int(n), rn));
+        if (xm::is_nan(err)) {
             n_rej += 1;
             status |= ODE_ST_NONFINITE;
             phase = PH_DONE;
             return;
         }
-        if (err > 1.0) {
+        const double lerr = xm::log_series(err);  // serves this step's powers and the next one's
+        if (xm::lt_nn(1.0, err)) {
             n_rej += 1;
-            h = 0.8 * h / xm::pow_series(err, 1.0 / 3.0);
+            h = 0.8 * h / xm::pow_log(lerr, 1.0 / 3.0);
             rejected = true;
             if (h < hmin) {
                 status |= ODE_ST_H_UNDERFLOW;
@@ -619,25 +643,37 @@ struct RkcF64 {
         t = t + h;
         num_step += 1;
         double fac = 10.0;
-        if (h_old < kUround) {
-            const double temp2 = xm::pow_series(err, 1.0 / 3.0);
-            if (0.8 < fac * temp2) fac = 0.8 / temp2;
+        if (xm::lt_nn(h_old, kUround)) {
+            const double temp2 = xm::pow_log(lerr, 1.0 / 3.0);
+            if (xm::lt_nn(0.8, fac * temp2)) fac = 0.8 / temp2;
         } else {
-            const double temp1 = 0.8 * h * xm::pow_series(err_old, 1.0 / 3.0);
-            const double temp2 = h_old * xm::pow_series(err, 2.0 / 3.0);
-            if (temp1 < fac * temp2) fac = temp1 / temp2;
+            // err_old^(1/3) and err^(2/3): in a team of lanes, one
+            // exponential with the two arguments on alternate lanes
+            double p1, p2;
+            if constexpr (W > 1) {
+                const double p = xm::pow_log((tm.lane & 1) ? lerr : lerr_old, (tm.lane & 1) ? 2.0 / 3.0 : 1.0 / 3.0);
+                p1 = tm.bcast(p, 0);
+                p2 = tm.bcast(p, 1);
+            } else {
+                p1 = xm::pow_log(lerr_old, 1.0 / 3.0);
+                p2 = xm::pow_log(lerr, 2.0 / 3.0);
+            }
+            const double temp1 = 0.8 * h * p1;
+            const double temp2 = h_old * p2;
+            if (xm::lt_nn(temp1, fac * temp2)) fac = temp1 / temp2;
         }
         err_old = err;
+        lerr_old = lerr;
         h_old = h;
         bool bad = false;
 #pragma unroll(P <= 64 ? P : 4)
         for (int s = 0; s < P; ++s) {
             yn[s] = w1[s];
             Fn[s] = f[s];
-            if (sys.comp(tm, s) >= 0 && !isfinite(w1[s])) bad = true;
+            if (sys.comp(tm, s) >= 0 && !xm::is_finite(w1[s])) bad = true;
         }
-        h = h * fmax(kP1, fac);
-        h = fmax(hmin, fmin(hmax, h));
+        h = h * xm::max_nn(kP1, fac);
+        h = xm::max_nn(hmin, xm::min_nn(hmax, h));
         if (tm.any(bad)) {
             status |= ODE_ST_NONFINITE;
             phase = PH_DONE;
