@@ -159,6 +159,9 @@ int validate_desc(const ode_rhs_desc* d, RhsEntry* r) {
         dv.insert(dv.end(), d->log10A, d->log10A + R);
         dv.insert(dv.end(), d->beta, d->beta + R);
         dv.insert(dv.end(), d->Ea, d->Ea + R);
+        for (int j = 0; j < R; ++j) dv.push_back(2.302585092994046 * d->log10A[j]);
+        for (int i = 0; i < S; ++i) dv.push_back(1.0 / d->mol_weights[i]);
+        for (int i = 0; i < S; ++i) dv.push_back(8.314462618 / d->mol_weights[i]);
         if (dv.size() % 2) dv.push_back(0.0);  // the float4 section starts 16-byte aligned
         std::vector<float> fv;
         const double log2_10 = 3.321928094887362, log2_e = 1.4426950408889634, r_gas = 8.314462618;
@@ -197,6 +200,9 @@ int validate_desc(const ode_rhs_desc* d, RhsEntry* r) {
         const size_t sched_pos = iv.size();
         for (int k = 0; k < sched_k; ++k)
             for (int l = 0; l < 32; ++l) iv.push_back(k < (int)lane_sp[l].size() ? lane_sp[l][k] : -1);
+        const size_t reac_pos = iv.size();
+        for (int j = 0; j < R; ++j)
+            iv.push_back(d->reac[2 * j] | (d->n_reac[j] == 2 ? d->reac[2 * j + 1] : kKinOne) << 8);
         const size_t dbytes = sizeof(double) * dv.size(), fbytes = sizeof(float) * fv.size(),
                      ibytes = sizeof(int) * iv.size();
         void* mem = nullptr;
@@ -222,11 +228,15 @@ int validate_desc(const ode_rhs_desc* d, RhsEntry* r) {
         kd.log10A = dp + 5 * S;
         kd.beta = kd.log10A + R;
         kd.Ea = kd.beta + R;
+        kd.ln10A = kd.Ea + R;
+        kd.rW = kd.ln10A + R;
+        kd.rgW = kd.rW + S;
         kd.rate32 = fp;
         kd.thermo32 = fp + R;
         kd.inc_off = ip;
         kd.inc = ip + S + 1;
         kd.sched = ip + sched_pos;
+        kd.reac = ip + reac_pos;
         kd.sched_k = sched_k;
         r->kin_alloc = mem;
         return ODE_OK;

@@ -106,6 +106,12 @@ struct KinDevice {
     const double* log10A;   // [R]
     const double* beta;
     const double* Ea;
+    // the plain form's constants of the mechanism, each the correctly
+    // rounded value its expression would take in every evaluation
+    const double* ln10A;    // [R] ln(10) log10 A
+    const double* rW;       // [S] 1 / W
+    const double* rgW;      // [S] R_gas / W
+    const int* reac;        // [R] first reactant | second << 8 (kKinOne: none)
     const int* inc_off;     // [S + 1]
     const int* inc;         // [inc_off[S]]
     const float4* rate32;   // [R]

@@ -1,0 +1,44 @@
+"""The plain FP64 kernels' own arrangements of the method against the oracle,
+bit for bit, at the sizes where an arrangement changes: kinetics mechanisms
+from a few species to the largest, and divisors outside the range that
+quotients by reciprocal take."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1611_02274_gb300 import binding as B
+from paper_1611_02274_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def assert_same(w, method, **kw):
+    import torch
+    h = B.register_workload(w)
+    try:
+        cnt = B.counters_like(w.nsys, "cuda")
+        y = B.integrate(method, h, torch.from_numpy(w.y0).cuda(), torch.from_numpy(w.params).cuda(), w.t0, w.tend,
+                        w.rtol, w.atol, counters=cnt, sync=True, **kw).cpu().numpy()
+    finally:
+        B.release(h)
+    r = O.integrate(O.model_for(w), {"rkck": W.METHOD_RKCK, "rkc": W.METHOD_RKC}[method], w.y0, w.params, w.t0, w.tend,
+                    w.rtol, w.atol)
+    np.testing.assert_array_equal(cnt.n_accept.cpu().numpy(), r.n_accept)
+    np.testing.assert_array_equal(cnt.n_rhs.cpu().numpy(), r.n_rhs)
+    np.testing.assert_array_equal(y, r.y)
+
+
+@pytest.mark.parametrize("species,reactions,density", [(12, 9, 1.0), (32, 33, 1.0), (33, 100, 1.0), (57, 766, 1.0),
+                                                       (62, 1000, 1.0), (57, 766, 1e-31)])
+def test_kinetics_sizes(species, reactions, density):
+    """Mechanisms around a warp's 32 lanes; a density below 2^-100 divides in full."""
+    mech = W.make_mechanism(3, species, reactions)
+    rng = np.random.default_rng(species + reactions)
+    n = 7
+    Y = rng.uniform(0.0, 1.0, (species, n)) * (rng.random((species, n)) < 0.6)  # absent species are exact zeros
+    Y[-1] += 0.1
+    Y /= Y.sum(axis=0)
+    y0 = np.concatenate([rng.uniform(1000.0, 1300.0, (1, n)), Y])
+    w = W.Workload("kinetics", W.RHS_KINETICS, W.METHOD_RKC, n, species + 1, np.ascontiguousarray(y0),
+                   np.full((1, n), 0.3 * density), 0.0, 2e-7, 1e-6, 1e-10, aux={"mechanism": mech})
+    assert_same(w, "rkc")
