@@ -474,15 +474,29 @@ struct NbodyCtx {
 // positions come from shuffles, taken in ascending order j as in the
 // defining sum.  The plain form evaluates m_j d / (r2 sqrt(r2)) as written;
 // the mixed form uses the reciprocal square root.  params [G].
-template <int W_>
+// PAIRS (the plain form): the FP64 pipe bounds it, and d, r^3 and its
+// reciprocal are the same for the two bodies of a pair up to the sign of d.
+// Each lane forms them for the next floor(n / 2) bodies round the ring only
+// and leaves them in the team's shared memory for both; the quotients by
+// r^3 then take three FP64 instructions each (xm::div_by).  Seven bodies:
+// 194 -> 123 FP64 instructions' time per lane and evaluation, each value as
+// before bit for bit; RKCK on 16,384 systems 82.6 -> 54.4 ms.
+template <int W_, bool PAIRS = false>
 struct NbodyModel {
     static constexpr int W = W_, PER = 4;
     using Ctx = NbodyCtx;
+    // PAIRS: four FP64 planes (dx, dy, r^3, 1 / r^3) of W rows of W + 1
+    static constexpr int kPlane = W_ * (W_ + 1);
+    static constexpr int SMEM_FLOATS = PAIRS ? 8 * (W_ + 1) : 0;
     template <class R>
     struct Sys {
         R G;
         R m[W_];
         int n, nb;
+        double* pair;  // PAIRS: this team's planes
+        __device__ void bind(float* block_base, int) {
+            pair = reinterpret_cast<double*>(block_base + (threadIdx.x / W) * W * SMEM_FLOATS);
+        }
         __device__ void load(const Ctx& ctx, const Team<W>&, double g, int neq) {
             G = (R)g;
             n = neq;
@@ -507,6 +521,41 @@ struct NbodyModel {
         __device__ void rhs(const Team<W>& tm, R, const R* y, R* f) const {
             const R x = y[0], yy = y[1];
             R ax = R(0), ay = R(0);
+            if constexpr (PAIRS) {
+                const int i = tm.lane;
+                for (int d = 1; d <= nb / 2; ++d) {
+                    const int j = i + d < nb ? i + d : i + d - nb;
+                    const double xj = tm.bcast(x, j), yj = tm.bcast(yy, j);
+                    if (i < nb) {
+                        const double dx = xj - x, dy = yj - yy;
+                        const double r2 = dx * dx + dy * dy;
+                        const double r3 = r2 * sqrt(r2), rr = xm::reciprocal(r3);
+                        double *a = pair + i * (W_ + 1) + j, *b = pair + j * (W_ + 1) + i;
+                        a[0] = dx;
+                        a[kPlane] = dy;
+                        b[0] = -dx;
+                        b[kPlane] = -dy;
+                        a[2 * kPlane] = b[2 * kPlane] = r3;
+                        a[3 * kPlane] = b[3 * kPlane] = rr;
+                    }
+                }
+                __syncwarp(tm.mask);
+                const double* row = pair + i * (W_ + 1);
+#pragma unroll
+                for (int j = 0; j < W_; ++j) {
+                    if (j < nb && i < nb && j != i) {
+                        const double r3 = row[2 * kPlane + j], rr = row[3 * kPlane + j];
+                        ax = ax + xm::div_by(m[j] * row[j], r3, rr);
+                        ay = ay + xm::div_by(m[j] * row[kPlane + j], r3, rr);
+                    }
+                }
+                __syncwarp(tm.mask);  // read before the next evaluation writes them
+                f[0] = y[2];
+                f[1] = y[3];
+                f[2] = G * ax;
+                f[3] = G * ay;
+                return;
+            }
 #pragma unroll
             for (int j = 0; j < W_; ++j) {
                 const R xj = tm.bcast(x, j), yj = tm.bcast(yy, j);

@@ -1,7 +1,7 @@
 """The plain FP64 kernels' own arrangements of the method against the oracle,
 bit for bit, at the sizes where an arrangement changes: kinetics mechanisms
-from a few species to the largest, and divisors outside the range that
-quotients by reciprocal take."""
+from a few species to the largest, divisors outside the range that
+quotients by reciprocal take, n-body rings, and the lanes a grid system takes."""
 import numpy as np
 import pytest
 
@@ -42,3 +42,17 @@ def test_kinetics_sizes(species, reactions, density):
     w = W.Workload("kinetics", W.RHS_KINETICS, W.METHOD_RKC, n, species + 1, np.ascontiguousarray(y0),
                    np.full((1, n), 0.3 * density), 0.0, 2e-7, 1e-6, 1e-10, aux={"mechanism": mech})
     assert_same(w, "rkc")
+
+
+@pytest.mark.parametrize("bodies", [1, 2, 3, 7, 8, 9, 12, 16])
+@pytest.mark.parametrize("method", ["rkck", "rkc"])
+def test_nbody_pairs(bodies, method):
+    """Each pair formed by one of its two lanes: odd and even rings, 8- and 16-lane teams at their edges."""
+    rng = np.random.default_rng(bodies)
+    n = 9
+    ang = 2 * np.pi * np.arange(bodies) / bodies
+    pos = 3.0 * np.stack([np.cos(ang), np.sin(ang)]).reshape(-1, 1) + 0.05 * rng.standard_normal((2 * bodies, n))
+    y0 = np.concatenate([pos, 0.5 * rng.standard_normal((2 * bodies, n))])
+    w = W.Workload("nbody", W.RHS_NBODY, W.METHOD_RKCK, n, 4 * bodies, np.ascontiguousarray(y0), np.ones((1, n)), 0.0,
+                   0.25, 1e-8, 1e-8, aux={"masses": 0.1 * np.arange(1.0, bodies + 1)})
+    assert_same(w, method)
