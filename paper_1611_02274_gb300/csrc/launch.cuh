@@ -26,7 +26,7 @@ struct RhsEntry {
 struct LaunchCfg {
     int mapping;     // ODE_MAP_THREAD or ODE_MAP_QUEUE
     int block;       // threads per block
-    int team;        // requested lanes per system (0 = family default)
+    int team;        // requested lanes per system (0 = family default; 32 keeps grids at a warp per system)
     int sm_count;
     cudaStream_t stream;
 };
@@ -62,6 +62,30 @@ cudaError_t launch_method(const BatchArgs& a, const Ctx& ctx, const LaunchCfg& c
 }
 
 enum { kMethodRkck = 0, kMethodRkc = 1 };
+
+// Lanes per system of the plain form's grid families (Brusselator grids,
+// oscillator chains).  The FP64 pipe bounds them, and a warp pays for an
+// FP64 instruction whatever its active lanes: the per-system part of a step
+// (controller, logarithm and powers, the norm's sequential sum) costs a warp
+// with four systems in it as much as a warp with one.  So where the batch
+// fills the GPU a system takes as few lanes as hold it at four points each
+// (more points a lane spill), and where it does not, a whole warp, which
+// has the shortest step.  Time is taken as rounds of warps over the SMs'
+// four sub-partitions times a step's FP64 work, in units of one point's:
+// G points a lane plus kOwn + kSum npts for the system (from the FP64
+// instruction counts of an RKC step: 150 a point, 110 a system and two per
+// point in the norm).  Measured on 32 points, wide / narrow: 8,192 systems
+// 68.3 / 52.5 ms.
+inline int grid_team_f64(int npts, int64_t nsys, int sm_count) {
+    constexpr double kOwn = 0.75, kSum = 0.0133;
+    int w = 1;
+    while (w < 32 && 4 * w < npts) w *= 2;
+    const int64_t slots = 4 * (int64_t)sm_count;
+    auto rounds = [&](int lanes) { return (double)(((nsys * lanes + 31) / 32 + slots - 1) / slots); };
+    const double system = kOwn + kSum * npts;
+    const double narrow = rounds(w) * (4.0 + system), wide = rounds(32) * ((npts + 31) / 32 + system);
+    return narrow < wide ? w : 32;
+}
 
 // Per-family dispatch (defined in k_*.cu).  Each sets *ok = false when the
 // family / size / precision / mapping combination is not built.

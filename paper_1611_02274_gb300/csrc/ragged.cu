@@ -89,7 +89,9 @@ cudaError_t launch_shape(int family, int method, int prec, const Shape& sh, cons
     if (sh.team == 0) {
         RhsEntry rr = r;
         rr.neq = sh.max_neq;  // size of the default kernel to use
-        return family == ODE_RHS_BRUSS1D ? launch_bruss(method, prec, rr, a, c, ok) : launch_chain(method, prec, rr, a, c, ok);
+        LaunchCfg warp = c;
+        warp.team = 32;  // the shape's meaning: a warp per system in every form
+        return family == ODE_RHS_BRUSS1D ? launch_bruss(method, prec, rr, a, warp, ok) : launch_chain(method, prec, rr, a, warp, ok);
     }
     if (prec == ODE_PREC_F2_LEAN)
         return family == ODE_RHS_BRUSS1D ? launch_bruss_shape_f2(sh.team, sh.g, a, g, c, ok)

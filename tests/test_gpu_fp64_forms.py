@@ -56,3 +56,20 @@ def test_nbody_pairs(bodies, method):
     w = W.Workload("nbody", W.RHS_NBODY, W.METHOD_RKCK, n, 4 * bodies, np.ascontiguousarray(y0), np.ones((1, n)), 0.0,
                    0.25, 1e-8, 1e-8, aux={"masses": 0.1 * np.arange(1.0, bodies + 1)})
     assert_same(w, method)
+
+
+@pytest.mark.parametrize("family", ["bruss", "chain"])
+@pytest.mark.parametrize("method", ["rkc", "rkck"])
+@pytest.mark.parametrize("points,nsys", [(1, 700), (4, 5000), (5, 3001), (8, 3000), (9, 2500), (16, 2500), (17, 1300),
+                                         (32, 1301), (33, 5), (33, 700), (64, 650), (40, 7)])
+def test_grid_shapes(family, method, points, nsys):
+    """Lanes per system by size and batch: both sides of each team width and of the wide kernels."""
+    if family == "bruss":
+        w = W.bruss(nsys=nsys, n=points, seed=points)
+        w.tend = 0.05
+    else:
+        rng = np.random.default_rng(points)
+        w = W.Workload("chain", W.RHS_VDP_CHAIN, W.METHOD_RKCK, nsys, 2 * points,
+                       rng.uniform(-2.0, 2.0, (2 * points, nsys)), 10.0 ** rng.uniform(-1.0, 1.0, (1, nsys)), 0.0, 0.2,
+                       1e-6, 1e-9)
+    assert_same(w, method)
