@@ -541,6 +541,7 @@ int integrate(Method method, int32_t handle, int64_t nsys, const double* y0, con
     a.tend = tend;
     a.rtol = rtol;
     a.atol = atol;
+    a.u = UniformScalars(t0, tend, rtol, atol);
     a.n_accept = d_stats.n_accept;
     a.n_reject = d_stats.n_reject;
     a.n_rhs = d_stats.n_rhs;

@@ -1,5 +1,6 @@
 // common.cuh -- shared device definitions of the batched integrators.
 #pragma once
+#include <cmath>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -141,6 +142,25 @@ struct BrussConst {
     double A, B, ubc, vbc;
 };
 
+// Step-size bounds, tolerances and the stage cap of one interval and
+// tolerance pair, in the widths the two-float RKC integrator uses.
+struct UniformScalars {
+    double hmax, hmin;
+    float hmaxf, hminf, rtolf, atolf;
+    int32_t mmax;
+    UniformScalars() = default;
+    __host__ __device__ UniformScalars(double t0, double tend, double rtol, double atol) {
+        hmax = fabs(tend - t0);
+        hmin = 10.0 * kUround * fmax(fabs(t0), fabs(tend - t0));
+        hmaxf = (float)hmax;
+        hminf = (float)hmin;
+        rtolf = (float)rtol;
+        atolf = (float)atol;
+        mmax = (int)round(sqrt(rtol / (10.0 * kUround)));
+        if (mmax < 2) mmax = 2;
+    }
+};
+
 // Everything one batched launch needs besides the model.
 struct MlpPacked;  // mlp_warp.cuh
 
@@ -209,6 +229,7 @@ struct BatchArgs {
     // pre_consts[j * pre_stride + i]); NULL = computed at each system's set-up
     const void* pre_consts;
     int64_t pre_stride;
+    UniformScalars u;  // of (t0, tend, rtol, atol), uniform batches
 
     __host__ __device__ int64_t sys_of(int64_t k) const { return index ? (int64_t)index[k] : k; }
     __host__ __device__ int64_t cidx(int64_t i, int w) const { return i + nsys * (int64_t)w; }

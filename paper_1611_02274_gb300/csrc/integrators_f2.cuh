@@ -60,26 +60,35 @@ template <class Model, bool BK64 = false, bool NET = false>
 struct RkcF2 {
     static constexpr bool kStepSync = true;  // variable stage count: hold at the step end
     static constexpr int W = Model::W, P = Model::PER;
+    // Register budget of the warp-wide kernels (they wait on the latency of
+    // the sums' chains, so warps count): one point a lane 128 instead of 141,
+    // 32-point grids, 65,536 systems 30.8 -> 28.3 ms; four points 168
+    // instead of 234, the mixed batch of 32,768 systems 64.6 -> 57.8 ms.
+    static constexpr int kMaxRegs = W == 32 ? (P == 2 ? 128 : P >= 8 ? 168 : 255) : 255;
     // the proposal network at the spectral-radius points (one thread per
     // system, up to 32 components + the parameter)
     using R = F2;
     using TM = Team<W>;
     using HT = typename Pick<BK64, double, float>::type;
     typename Model::template Sys<F2> sys;
-    F2 Fn[P], d1[P];  // d_j = w_j - y_n (d_0 = 0); y_n and d_{j-2} below
+    // Slots i and i + NP share a pack (F2x2): the element-wise work of a step
+    // runs on the packed FP32 instructions, half as many as one slot at a
+    // time; an odd P leaves the last pack's second half at zero.
+    static constexpr int NP = (P + 1) / 2;
+    F2x2 Fn[NP], d1[NP];  // d_j = w_j - y_n (d_0 = 0); y_n and d_{j-2} below
     static constexpr int V_SMEM = rkc_f2_smem_floats(W, P);
     // the system's constants, one row per thread after the V rows (an even
     // offset: 8-byte aligned pairs, since blocks are a multiple of 32 threads)
     static constexpr int C_SMEM = ConstSmem<typename Model::template Sys<F2>>::value;
     // d_{j-2}, needed only from the third stage on: for one-thread systems a
-    // row of pairs in shared memory (an odd number of pairs per row), so a
-    // two-stage step -- the common case at tight tolerances -- touches it
-    // never and holds no registers for it
-    static constexpr int D2_SMEM = (W == 1 && P <= 32) ? 2 * (P | 1) : 0;
+    // row of packs in shared memory (an odd number of 16-byte packs per row:
+    // no bank conflicts), so a two-stage step -- the common case at tight
+    // tolerances -- touches it never and holds no registers for it
+    static constexpr int D2_SMEM = (W == 1 && P <= 32) ? 4 * (NP | 1) : 0;
     // the state y_n, read at the evaluation points, the error weights and
     // the accept only: for one-thread systems a shared-memory row too, so
     // that no state pair stays live across the right-hand-side evaluation
-    static constexpr int Y_SMEM = (W == 1 && P <= 32) ? 2 * (P | 1) : 0;
+    static constexpr int Y_SMEM = D2_SMEM;
     static constexpr int SMEM_FLOATS = V_SMEM + C_SMEM + D2_SMEM + Y_SMEM + ModelSmem<Model>::value;
     // the proposal network at the spectral-radius points (one thread per
     // system with rows in shared memory: up to 32 components + the
@@ -88,50 +97,71 @@ struct RkcF2 {
     static constexpr bool kWarpPropose = NET && W == 1 && P <= 32 && D2_SMEM >= 8 * kMlpKs && Y_SMEM > 0;
     static constexpr int kJoin = 12;  // steps before its point a system joins a warp's network evaluation
     mutable F2 vreg[V_SMEM ? 1 : P];
-    mutable F2 d2reg[D2_SMEM ? 1 : P];
-    mutable F2 yreg[Y_SMEM ? 1 : P];
+    mutable F2x2 d2reg[D2_SMEM ? 1 : NP];
+    mutable F2x2 yreg[Y_SMEM ? 1 : NP];
     float* vs;
-    F2* d2s;
-    F2* ys;
+    float* d2s;
+    float* ys;
     __device__ void bind_smem(float* base, int stride) {
         vs = base + threadIdx.x * V_SMEM;  // this thread's row
         if constexpr (C_SMEM > 0) sys.bind_consts(base + V_SMEM * stride + threadIdx.x * C_SMEM);
-        if constexpr (D2_SMEM > 0)
-            d2s = reinterpret_cast<F2*>(base + (V_SMEM + C_SMEM) * stride + threadIdx.x * D2_SMEM);
-        if constexpr (Y_SMEM > 0)
-            ys = reinterpret_cast<F2*>(base + (V_SMEM + C_SMEM + D2_SMEM) * stride + threadIdx.x * Y_SMEM);
+        // 16-byte rows: the offsets before them are multiples of 128 bytes
+        // (blocks are a multiple of 32 threads)
+        if constexpr (D2_SMEM > 0) d2s = base + (V_SMEM + C_SMEM) * stride + threadIdx.x * D2_SMEM;
+        if constexpr (Y_SMEM > 0) ys = base + (V_SMEM + C_SMEM + D2_SMEM) * stride + threadIdx.x * Y_SMEM;
         if constexpr (ModelSmem<Model>::value > 0)
             sys.bind(base + (V_SMEM + C_SMEM + D2_SMEM + Y_SMEM) * stride, stride);
     }
+    // packs of a shared-memory row: (hi, hi, lo, lo)
+    __device__ static F2x2 row_get(const float* row, int i) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + 4 * i);
+        return F2x2(v.x, v.y);
+    }
+    __device__ static void row_set(float* row, int i, F2x2 v) {
+        *reinterpret_cast<ulonglong2*>(row + 4 * i) = make_ulonglong2(v.hi, v.lo);
+    }
+    __device__ F2x2 Yp(int i) const {
+        if constexpr (Y_SMEM > 0)
+            return row_get(ys, i);
+        else
+            return yreg[i];
+    }
+    __device__ void Yset(int i, F2x2 v) const {
+        if constexpr (Y_SMEM > 0)
+            row_set(ys, i, v);
+        else
+            yreg[i] = v;
+    }
+    // one slot of a pack array
+    __device__ static F2 slot(F2x2 v, int s) { return s < NP ? v.first() : v.second(); }
     __device__ F2 Yg(int s) const {
-        if constexpr (Y_SMEM > 0)
-            return ys[s];
-        else
-            return yreg[s];
+        if constexpr (Y_SMEM > 0) {
+            const float* q = ys + 4 * (s % NP) + s / NP;
+            return F2(q[0], q[2]);
+        } else {
+            return slot(yreg[s % NP], s);
+        }
     }
-    __device__ void Ys(int s, F2 v) const {
-        if constexpr (Y_SMEM > 0)
-            ys[s] = v;
-        else
-            yreg[s] = v;
+    __device__ F2 Fg(int s) const { return slot(Fn[s % NP], s); }
+    // slots i and i + NP of a slot array; the half past the last slot is zero
+    __device__ static F2x2 both(const F2* x, int i) {
+        return F2x2(x[i], i + NP < P ? x[i + NP < P ? i + NP : i] : F2(0.0f, 0.0f));
     }
-    __device__ const F2* yp() const {
-        if constexpr (Y_SMEM > 0)
-            return ys;
-        else
-            return yreg;
+    __device__ static void split(F2x2 v, F2* x, int i) {
+        x[i] = v.first();
+        if (i + NP < P) x[i + NP] = v.second();
     }
-    __device__ F2 D2g(int s) const {
+    __device__ F2x2 D2g(int i) const {
         if constexpr (D2_SMEM > 0)
-            return d2s[s];
+            return row_get(d2s, i);
         else
-            return d2reg[s];
+            return d2reg[i];
     }
-    __device__ void D2s(int s, F2 v) const {
+    __device__ void D2set(int i, F2x2 v) const {
         if constexpr (D2_SMEM > 0)
-            d2s[s] = v;
+            row_set(d2s, i, v);
         else
-            d2reg[s] = v;
+            d2reg[i] = v;
     }
     __device__ F2 Vg(int s) const {
         if constexpr (V_SMEM > 0)
@@ -147,14 +177,39 @@ struct RkcF2 {
             vreg[s] = v;
         }
     }
+    __device__ HT gershgorin(const TM& tm) const {
+        F2 y[P];
+#pragma unroll(P <= 64 ? P : 4)
+        for (int s = 0; s < P; ++s) y[s] = Yg(s);
+        return (HT)to_double(sys.gershgorin(tm, y));
+    }
     double t, tend;                   // BK64
     float remf, reml, tendf;          // FP32 scalars: remaining interval as a pair
-    HT hmax, hmin, h, h_old, sigma;
+    HT hmax_, hmin_, h, h_old, sigma;
     F2 hh;                            // the step size as a pair (exact for an FP32 h)
-    float rtolf, atolf, c3_old, dynrm, sig;
-    float4 chi, clo;                  // (mu_j, nu_j, mu~_j, gamma~_j), leading / trailing words
-    CoefSource cs;
-    int32_t n_acc, n_rej, n_rhs, n_sr, status, max_att, mmax, num_step, sr_step, n;
+    float rtolf_, atolf_, c3_old, dynrm, sig;
+    int32_t n_acc, n_rej, n_rhs, n_sr, status, mmax_, num_step, sr_step, n_;
+    // One-thread systems come in uniform batches (ragged plans give a system
+    // a team), so the interval's and tolerances' scalars are kernel
+    // arguments, read where a step needs them (the host converts them once);
+    // stage coefficients are read from the table where they are used.  What
+    // stays in registers across the right-hand-side evaluation decides what
+    // the compiler spills: 472 -> 120 bytes in the 13-species kernel at its
+    // 168 registers, 1M systems in cost order 131.2 -> 118.7 ms (with the
+    // packed arithmetic).
+    static constexpr bool kUniform = W == 1;
+    __device__ HT hmax(const BatchArgs& a) const { return kUniform ? pick_ht(a.u.hmax, a.u.hmaxf) : hmax_; }
+    __device__ HT hmin(const BatchArgs& a) const { return kUniform ? pick_ht(a.u.hmin, a.u.hminf) : hmin_; }
+    __device__ float rtolf(const BatchArgs& a) const { return kUniform ? a.u.rtolf : rtolf_; }
+    __device__ float atolf(const BatchArgs& a) const { return kUniform ? a.u.atolf : atolf_; }
+    __device__ int mmax(const BatchArgs& a) const { return kUniform ? a.u.mmax : mmax_; }
+    __device__ int neq(const BatchArgs& a) const { return kUniform ? a.neq : n_; }
+    __device__ static HT pick_ht(double d, float f) {
+        if constexpr (BK64)
+            return d;
+        else
+            return f;
+    }
     int32_t phase, m, j, sr_iter;
     bool have_sigma, rejected, warm;
 
@@ -167,26 +222,28 @@ struct RkcF2 {
         } else {
             sys.load(ctx, tm, a.params[i], a.neq_of(i));
         }
-        n = a.neq_of(i);
+        n_ = a.neq_of(i);
+        auto y0 = [&](int s) {
+            const int c = s < P ? sys.comp(tm, s) : -1;
+            return F2(c >= 0 ? a.y0[a.yidx(i, c)] : 0.0);
+        };
 #pragma unroll(P <= 64 ? P : 4)
-        for (int s = 0; s < P; ++s) {
-            const int c = sys.comp(tm, s);
-            Ys(s, F2(c >= 0 ? a.y0[a.yidx(i, c)] : 0.0));
-        }
+        for (int q = 0; q < NP; ++q) Yset(q, F2x2(y0(q), y0(q + NP)));
         t = a.t0_of(i);
         tend = a.tend_of(i);
         remf = (float)(tend - t);
         reml = (float)((tend - t) - (double)remf);
         tendf = (float)tend;
-        rtolf = (float)a.rtol_of(i);
-        atolf = (float)a.atol_of(i);
-        mmax = (int)round(sqrt(a.rtol_of(i) / (10.0 * kUround)));
-        if (mmax < 2) mmax = 2;
-        hmax = (HT)fabs(tend - t);
-        hmin = (HT)(10.0 * kUround * fmax(fabs(t), fabs(tend - t)));
+        if constexpr (!kUniform) {
+            const UniformScalars u(t, tend, a.rtol_of(i), a.atol_of(i));
+            rtolf_ = u.rtolf;
+            atolf_ = u.atolf;
+            mmax_ = u.mmax;
+            hmax_ = pick_ht(u.hmax, u.hmaxf);
+            hmin_ = pick_ht(u.hmin, u.hminf);
+        }
         n_acc = n_rej = n_sr = status = 0;
         n_rhs = 1;
-        max_att = a.max_attempts;
         h = h_old = sigma = (HT)0;
         c3_old = 0.0f;
         num_step = 0;
@@ -220,8 +277,8 @@ struct RkcF2 {
             const float hp = a.h0[i], sp = a.sigma0[i];
             if (isfinite(sp) && sp > 0.0f) {
                 if (isfinite(hp) && hp > 0.0f) {
-                    h = (HT)hp < hmax ? (HT)hp : hmax;
-                    h = h > hmin ? h : hmin;
+                    h = (HT)hp < hmax(a) ? (HT)hp : hmax(a);
+                    h = h > hmin(a) ? h : hmin(a);
                 }
                 sigma = (HT)sp;
                 have_sigma = true;
@@ -264,11 +321,11 @@ struct RkcF2 {
             break;
         case PH_TRIAL:
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) x[s] = Yg(s) + hh * Fn[s];
+            for (int q = 0; q < NP; ++q) split(Yp(q) + F2x2(hh) * Fn[q], x, q);
             break;
         default:  // stages and F_{n+1}: w = y_n + d (left unnormalised: it feeds products)
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) x[s] = add_lazy(Yg(s), d1[s]);
+            for (int q = 0; q < NP; ++q) split(add_lazy(Yp(q), d1[q]), x, q);
         }
     }
 
@@ -276,15 +333,16 @@ struct RkcF2 {
         switch (phase) {
         case PH_F0:
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) {
-                Fn[s] = f[s];
-                if (!warm) Vs(s, f[s]);  // first eigenvector guess
+            for (int q = 0; q < NP; ++q) Fn[q] = both(f, q);
+            if (!warm) {
+#pragma unroll(P <= 64 ? P : 4)
+                for (int s = 0; s < P; ++s) Vs(s, f[s]);  // first eigenvector guess
             }
             loop_top(a, tm);
             break;
         case PH_SR: sr_consume(a, tm, f); break;
         case PH_TRIAL: trial_consume(a, tm, f); break;
-        case PH_STAGE: stage_consume(f); break;
+        case PH_STAGE: stage_consume(a, f); break;
         default: final_consume(a, tm, x, f);
         }
         return done();
@@ -302,7 +360,7 @@ struct RkcF2 {
                 return;
             }
         }
-        if (n_acc + n_rej >= max_att) {
+        if (n_acc + n_rej >= a.max_attempts) {
             status |= ODE_ST_MAX_ATTEMPTS;
             phase = PH_DONE;
             return;
@@ -335,7 +393,7 @@ struct RkcF2 {
         }
         if (!have_sigma || rejected || (num_step % kSpecradEvery == 0 && sr_step != num_step)) {
             if (a.specrad == ODE_SPECRAD_GERSHGORIN) {  // the bound replaces the power method
-                sigma = (HT)to_double(sys.gershgorin(tm, yp()));
+                sigma = gershgorin(tm);
                 have_sigma = true;
                 sr_step = num_step;
                 after_sr(a);
@@ -380,8 +438,8 @@ struct RkcF2 {
 #pragma unroll 1
                 for (int k = 0; k < 16 * kMlpKs; ++k) {
                     float fx = 0.0f;
-                    if (k <= n) {
-                        const float raw = k < n ? __logf(fmaxf(fabsf(ys[k].hi), 1e-30f)) : par;
+                    if (k <= neq(a)) {
+                        const float raw = k < neq(a) ? __logf(fmaxf(fabsf(ys[4 * (k % NP) + k / NP]), 1e-30f)) : par;
                         fx = (raw - net->x_mean[k]) * net->x_iscale[k];
                         inside = inside && raw >= net->x_lo[k] && raw <= net->x_hi[k];
                     }
@@ -448,13 +506,13 @@ struct RkcF2 {
         float acc = 0.0f;
 #pragma unroll(P <= 64 ? P : 4)
         for (int s = 0; s < P; ++s) {
-            df[s] = Fv[s] - Fn[s];
+            df[s] = Fv[s] - Fg(s);
             if (sys.comp(tm, s) >= 0) acc = fmaf(df[s].hi, df[s].hi, acc);
         }
         const float d = sqrtf(tm.sum(acc));
         const float sig_prev = sig;
         sig = d / dynrm;
-        if (sr_iter >= 2 && fabsf(sig - sig_prev) <= fmaxf(sig, 1.0f / (float)hmax) * 0.01f) {
+        if (sr_iter >= 2 && fabsf(sig - sig_prev) <= fmaxf(sig, 1.0f / (float)hmax(a)) * 0.01f) {
 #pragma unroll(P <= 64 ? P : 4)
             for (int s = 0; s < P; ++s) Vs(s, Vg(s) - Yg(s));
             sr_end(a, tm);
@@ -465,7 +523,7 @@ struct RkcF2 {
 #pragma unroll(P <= 64 ? P : 4)
             for (int s = 0; s < P; ++s) Vs(s, Yg(s) + df[s] * sc);
         } else {
-            const int ind = sr_iter % n;
+            const int ind = sr_iter % neq(a);
 #pragma unroll(P <= 64 ? P : 4)
             for (int s = 0; s < P; ++s)
                 if (opaque(sys.comp(tm, s)) == ind) Vs(s, Yg(s) - (Vg(s) - Yg(s)));
@@ -481,7 +539,7 @@ struct RkcF2 {
     __device__ void sr_end(const BatchArgs& a, const TM& tm) {
         sigma = (HT)1.2 * (HT)sig;
         if (a.specrad == ODE_SPECRAD_POWER_CAPPED) {
-            const HT g = (HT)to_double(sys.gershgorin(tm, yp()));
+            const HT g = gershgorin(tm);
             sigma = sigma < g ? sigma : g;
         }
         have_sigma = true;
@@ -491,9 +549,9 @@ struct RkcF2 {
 
     __device__ void after_sr(const BatchArgs& a) {
         if (h < (HT)kUround) {
-            h = hmax;
+            h = hmax(a);
             if (sigma * h > (HT)1) h = (HT)1 / sigma;
-            h = h > hmin ? h : hmin;
+            h = h > hmin(a) ? h : hmin(a);
             hh = F2(h);
             phase = PH_TRIAL;
             return;
@@ -520,31 +578,31 @@ struct RkcF2 {
     __device__ void trial_consume(const BatchArgs& a, const TM& tm, const F2* f) {
         n_rhs += 1;
         const HT ssq = weighted_ssq(tm, [&](int s) {
-            return __fdividef(to_float(f[s] - Fn[s]), atolf + rtolf * fabsf(Yg(s).hi));
+            return __fdividef(to_float(f[s] - Fg(s)), atolf(a) + rtolf(a) * fabsf(Yg(s).hi));
         });
-        const HT est = h * sqrt(ssq / (HT)n);
-        if ((HT)kP1 * h < hmax * sqrt(est)) {
+        const HT est = h * sqrt(ssq / (HT)neq(a));
+        if ((HT)kP1 * h < hmax(a) * sqrt(est)) {
             h = (HT)kP1 * h / sqrt(est);
-            h = h > hmin ? h : hmin;
+            h = h > hmin(a) ? h : hmin(a);
         } else {
-            h = hmax;
+            h = hmax(a);
         }
         stage_begin(a);
     }
 
     __device__ void stage_begin(const BatchArgs& a) {
         m = 1 + (int)sqrt((HT)1.54 * h * sigma + (HT)1);
-        if (m > mmax) {
-            m = mmax;
+        if (m > mmax(a)) {
+            m = mmax(a);
             h = (HT)(m * m - 1) / ((HT)1.54 * sigma);
         }
         hh = F2(h);
+        CoefSource cs;
         cs.start(m, a);
-        const F2 mut1h = cs.mut1f2() * hh;
+        const F2x2 mut1h(cs.mut1f2() * hh);
 #pragma unroll(P <= 64 ? P : 4)
-        for (int s = 0; s < P; ++s) d1[s] = mul_lazy(mut1h, Fn[s]);  // a product: its pair stays near-normal
+        for (int q = 0; q < NP; ++q) d1[q] = mul_lazy(mut1h, Fn[q]);  // a product: its pair stays near-normal
         j = 2;
-        cs.stagef2(2, chi, clo);
         phase = PH_STAGE;
     }
 
@@ -558,36 +616,38 @@ struct RkcF2 {
     // coefficient once per step, two products and one sum per component
     // (the two-stage step is the one every system takes at tight
     // tolerances).
-    __device__ void stage_consume(const F2* f) {
-        const F2 mu(chi.x, clo.x), nu(chi.y, clo.y);
-        const F2 muth = F2(chi.z, clo.z) * hh;
+    __device__ void stage_consume(const BatchArgs& a, const F2* f) {
+        float4 chi, clo;  // (mu_j, nu_j, mu~_j, gamma~_j), leading / trailing words
+        CoefSource cs;
+        cs.start(m, a);
+        cs.stagef2(j, chi, clo);
+        const F2 mu(chi.x, clo.x);
+        const F2x2 muth(F2(chi.z, clo.z) * hh);
         const bool keep = j < m;  // d_{j-1} is the next stage's d_{j-2}
         if (j == 2) {
-            const F2 c2h = (mu * cs.mut1f2() + F2(chi.w, clo.w)) * hh;
+            const F2x2 c2h((mu * cs.mut1f2() + F2(chi.w, clo.w)) * hh);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) {
-                const F2 dj = add_lazy(mul_lazy(c2h, Fn[s]), mul_lazy(muth, f[s]));
-                if (keep) D2s(s, d1[s]);
-                d1[s] = dj;
+            for (int q = 0; q < NP; ++q) {
+                const F2x2 dj = add_lazy(mul_lazy(c2h, Fn[q]), mul_lazy(muth, both(f, q)));
+                if (keep) D2set(q, d1[q]);
+                d1[q] = dj;
             }
         } else {
-            const F2 gth = F2(chi.w, clo.w) * hh;
+            const F2x2 mup(mu), nu(F2(chi.y, clo.y)), gth(F2(chi.w, clo.w) * hh);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) {
-                const F2 dj = add_lazy(
-                    add_lazy(add_lazy(mul_lazy(mu, d1[s]), mul_lazy(nu, D2g(s))), mul_lazy(muth, f[s])),
-                    mul_lazy(gth, Fn[s]));
-                if (keep) D2s(s, d1[s]);
-                d1[s] = dj;
+            for (int q = 0; q < NP; ++q) {
+                const F2x2 dj = add_lazy(
+                    add_lazy(add_lazy(mul_lazy(mup, d1[q]), mul_lazy(nu, D2g(q))), mul_lazy(muth, both(f, q))),
+                    mul_lazy(gth, Fn[q]));
+                if (keep) D2set(q, d1[q]);
+                d1[q] = dj;
             }
         }
         j += 1;
-        if (j <= m)
-            cs.stagef2(j, chi, clo);
-        else
-            phase = PH_FINAL;
+        if (j > m) phase = PH_FINAL;
     }
 
+    __device__ static constexpr int i_second(int q) { return q + NP; }
     // x = w_m (the point F_{n+1} was evaluated at), f = F_{n+1}.
     // Eq. E:rmsE's 0.8 (y_n - y_{n+1}) + 0.4 h (F_n + F_{n+1}) is computed as
     // 0.4 (h (F_n + F_{n+1}) - 2 d_m): the two terms cancel, so the leading
@@ -595,15 +655,24 @@ struct RkcF2 {
     // before the single rounding to FP32.
     __device__ void final_consume(const BatchArgs& a, const TM& tm, const F2* x, const F2* f) {
         n_rhs += m;
-        const HT ms = weighted_ssq(tm, [&](int s) {
-            const F2 sum = add_lazy(Fn[s], f[s]);  // feeds the product below: left unnormalised
-            const float p = hh.hi * sum.hi;
-            float e = fmaf(hh.hi, sum.hi, -p);
-            e = fmaf(hh.hi, sum.lo, e);
-            e = fmaf(hh.lo, sum.hi, e);
-            const float D = fmaf(-2.0f, d1[s].hi, p) + fmaf(-2.0f, d1[s].lo, e);
-            return __fdividef(0.4f * D, atolf + rtolf * fmaxf(fabsf(x[s].hi), fabsf(Yg(s).hi)));
-        }) / (HT)n;  // err^2
+        // error components e over their weights, both halves of a pack at
+        // once; the squares are then summed in slot order
+        float ew[2 * NP];
+        const f32x2 hhi = pack2(hh.hi, hh.hi), hlo = pack2(hh.lo, hh.lo), m2 = pack2(-2.0f, -2.0f);
+#pragma unroll(P <= 64 ? P : 4)
+        for (int q = 0; q < NP; ++q) {
+            const F2x2 sum = add_lazy(Fn[q], both(f, q));  // feeds the product below: left unnormalised
+            const f32x2 p = mul2(hhi, sum.hi);
+            f32x2 e = fma2(hhi, sum.hi, neg2(p));
+            e = fma2(hhi, sum.lo, e);
+            e = fma2(hlo, sum.hi, e);
+            const f32x2 D = mul2(pack2(0.4f, 0.4f), add2(fma2(m2, d1[q].hi, p), fma2(m2, d1[q].lo, e)));
+            const f32x2 y = Yp(q).hi;
+            const float x1 = i_second(q) < P ? x[i_second(q)].hi : 0.0f;
+            ew[q] = __fdividef(half0(D), fmaf(rtolf(a), fmaxf(fabsf(x[q].hi), fabsf(half0(y))), atolf(a)));
+            ew[q + NP] = __fdividef(half1(D), fmaf(rtolf(a), fmaxf(fabsf(x1), fabsf(half1(y))), atolf(a)));
+        }
+        const HT ms = weighted_ssq(tm, [&](int s) { return ew[s]; }) / (HT)neq(a);  // err^2
         if (isnan(ms)) {
             n_rej += 1;
             status |= ODE_ST_NONFINITE;
@@ -616,7 +685,7 @@ struct RkcF2 {
             n_rej += 1;
             h = h * (HT)(0.8f / c3);
             rejected = true;
-            if (h < hmin) {
+            if (h < hmin(a)) {
                 status |= ODE_ST_H_UNDERFLOW;
                 phase = PH_DONE;
                 return;
@@ -646,16 +715,18 @@ struct RkcF2 {
         }
         float chk = 0.0f;  // one finiteness test of a sum per system
 #pragma unroll(P <= 64 ? P : 4)
-        for (int s = 0; s < P; ++s) {
-            const F2 yn = Yg(s) + d1[s];
-            Ys(s, yn);
-            Fn[s] = f[s];
-            chk += (sys.comp(tm, s) >= 0) ? yn.hi - yn.hi : 0.0f;
+        for (int q = 0; q < NP; ++q) {
+            const F2x2 yn = Yp(q) + d1[q];
+            Yset(q, yn);
+            Fn[q] = both(f, q);
+            const f32x2 z = sub2(yn.hi, yn.hi);
+            chk += (sys.comp(tm, q) >= 0) ? half0(z) : 0.0f;
+            if (q + NP < P) chk += (sys.comp(tm, q + NP) >= 0) ? half1(z) : 0.0f;
         }
         const bool bad = !(chk == 0.0f);
         h = h * (HT)fmaxf((float)kP1, fac);
-        h = h < hmax ? h : hmax;
-        h = h > hmin ? h : hmin;
+        h = h < hmax(a) ? h : hmax(a);
+        h = h > hmin(a) ? h : hmin(a);
         if (tm.any(bad)) {
             status |= ODE_ST_NONFINITE;
             phase = PH_DONE;
@@ -668,8 +739,8 @@ struct RkcF2 {
 #pragma unroll(P <= 64 ? P : 4)
         for (int s = 0; s < P; ++s) {
             const int c = sys.comp(tm, s);
-            if (c >= 0) a.y_out[a.yidx_out(i, c)] = to_double(Yg(s));
             if (a.carry != nullptr && c >= 0) a.carry[a.cidx(i, kCarryFixed + c)] = to_double(Vg(s));
+            if (c >= 0) a.y_out[a.yidx_out(i, c)] = to_double(Yg(s));
         }
         if (a.carry != nullptr && tm.lane == 0) {
             const int st = status & 0xFF;
@@ -732,7 +803,17 @@ struct RkckF2 {
     using TM = Team<W>;
     using HT = typename Pick<BK64, double, float>::type;
     typename Model::template Sys<F2> sys;
-    F2 y[P], k1[P], k2[P], k3[P], k4[P], k5[P];
+    // slots i and i + NP share a pack, as in RkcF2
+    static constexpr int NP = (P + 1) / 2;
+    F2x2 y[NP], k1[NP], k2[NP], k3[NP], k4[NP], k5[NP];
+    __device__ static F2x2 both(const F2* x, int i) {
+        return F2x2(x[i], i + NP < P ? x[i + NP < P ? i + NP : i] : F2(0.0f, 0.0f));
+    }
+    __device__ static void split(F2x2 v, F2* x, int i) {
+        x[i] = v.first();
+        if (i + NP < P) x[i + NP] = v.second();
+    }
+    __device__ static F2x2 mulc(F2 c, F2x2 k) { return mul_lazy(F2x2(c), k); }
     double t, tend;                          // BK64
     HT h, hmax;
     F2 hh;                                   // the step size as a pair
@@ -741,11 +822,12 @@ struct RkckF2 {
 
     __device__ void init(const BatchArgs& a, const typename Model::Ctx& ctx, const TM& tm, int64_t i) {
         sys.load(ctx, tm, a.params[i], a.neq_of(i));
+        auto y0 = [&](int s) {
+            const int c = s < P ? sys.comp(tm, s) : -1;
+            return F2(c >= 0 ? a.y0[a.yidx(i, c)] : 0.0);
+        };
 #pragma unroll(P <= 64 ? P : 4)
-        for (int s = 0; s < P; ++s) {
-            const int c = sys.comp(tm, s);
-            y[s] = F2(c >= 0 ? a.y0[a.yidx(i, c)] : 0.0);
-        }
+        for (int q = 0; q < NP; ++q) y[q] = F2x2(y0(q), y0(q + NP));
         t = a.t0_of(i);
         tend = a.tend_of(i);
         hmax = (HT)fabs(tend - t);
@@ -799,40 +881,40 @@ struct RkckF2 {
         case 1:
             tx = F2(tb);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) x[s] = y[s];
+            for (int q = 0; q < NP; ++q) split(y[q], x, q);
             break;
         case 2:
             tx = F2(tb + (float)ck::A2 * hf);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) x[s] = add_lazy(y[s], mul_lazy(ck2::B21, k1[s]));
+            for (int q = 0; q < NP; ++q) split(add_lazy(y[q], mulc(ck2::B21, k1[q])), x, q);
             break;
         case 3:
             tx = F2(tb + (float)ck::A3 * hf);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s)
-                x[s] = add_lazy(y[s], add_lazy(mul_lazy(ck2::B31, k1[s]), mul_lazy(ck2::B32, k2[s])));
+            for (int q = 0; q < NP; ++q)
+                split(add_lazy(y[q], add_lazy(mulc(ck2::B31, k1[q]), mulc(ck2::B32, k2[q]))), x, q);
             break;
         case 4:
             tx = F2(tb + (float)ck::A4 * hf);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s)
-                x[s] = add_lazy(y[s], add_lazy(add_lazy(mul_lazy(ck2::B41, k1[s]), mul_lazy(ck2::B42, k2[s])),
-                                               mul_lazy(ck2::B43, k3[s])));
+            for (int q = 0; q < NP; ++q)
+                split(add_lazy(y[q], add_lazy(add_lazy(mulc(ck2::B41, k1[q]), mulc(ck2::B42, k2[q])),
+                                               mulc(ck2::B43, k3[q]))), x, q);
             break;
         case 5:
             tx = F2(tb + (float)ck::A5 * hf);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s)
-                x[s] = add_lazy(y[s], add_lazy(add_lazy(mul_lazy(ck2::B51, k1[s]), mul_lazy(ck2::B52, k2[s])),
-                                               add_lazy(mul_lazy(ck2::B53, k3[s]), mul_lazy(ck2::B54, k4[s]))));
+            for (int q = 0; q < NP; ++q)
+                split(add_lazy(y[q], add_lazy(add_lazy(mulc(ck2::B51, k1[q]), mulc(ck2::B52, k2[q])),
+                                               add_lazy(mulc(ck2::B53, k3[q]), mulc(ck2::B54, k4[q])))), x, q);
             break;
         default:
             tx = F2(tb + (float)ck::A6 * hf);
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s)
-                x[s] = add_lazy(y[s], add_lazy(add_lazy(add_lazy(mul_lazy(ck2::B61, k1[s]), mul_lazy(ck2::B62, k2[s])),
-                                                        add_lazy(mul_lazy(ck2::B63, k3[s]), mul_lazy(ck2::B64, k4[s]))),
-                                               mul_lazy(ck2::B65, k5[s])));
+            for (int q = 0; q < NP; ++q)
+                split(add_lazy(y[q], add_lazy(add_lazy(add_lazy(mulc(ck2::B61, k1[q]), mulc(ck2::B62, k2[q])),
+                                                        add_lazy(mulc(ck2::B63, k3[q]), mulc(ck2::B64, k4[q]))),
+                                               mulc(ck2::B65, k5[q]))), x, q);
         }
     }
 
@@ -840,23 +922,23 @@ struct RkckF2 {
         switch (stage) {
         case 1:
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) k1[s] = f[s] * hh;
+            for (int q = 0; q < NP; ++q) k1[q] = both(f, q) * F2x2(hh);
             break;
         case 2:
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) k2[s] = f[s] * hh;
+            for (int q = 0; q < NP; ++q) k2[q] = both(f, q) * F2x2(hh);
             break;
         case 3:
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) k3[s] = f[s] * hh;
+            for (int q = 0; q < NP; ++q) k3[q] = both(f, q) * F2x2(hh);
             break;
         case 4:
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) k4[s] = f[s] * hh;
+            for (int q = 0; q < NP; ++q) k4[q] = both(f, q) * F2x2(hh);
             break;
         case 5:
 #pragma unroll(P <= 64 ? P : 4)
-            for (int s = 0; s < P; ++s) k5[s] = f[s] * hh;
+            for (int q = 0; q < NP; ++q) k5[q] = both(f, q) * F2x2(hh);
             break;
         default:
             finish(tm, f);
@@ -869,22 +951,27 @@ struct RkckF2 {
     // fifth-order solution, embedded error (Section 2.1) and the step-size
     // rule of the listing
     __device__ void finish(const TM& tm, const F2* f) {
-        F2 yt[P];
+        F2x2 yt[NP];
         float err = 0.0f;
         bool nan_flag = false;
-#pragma unroll(P <= 64 ? P : 4)
-        for (int s = 0; s < P; ++s) {
-            const F2 k6 = f[s] * hh;
-            const F2 incr = add_lazy(add_lazy(mul_lazy(ck2::C1, k1[s]), mul_lazy(ck2::C3, k3[s])),
-                                     add_lazy(mul_lazy(ck2::C4, k4[s]), mul_lazy(ck2::C6, k6)));
-            yt[s] = y[s] + incr;
-            const float ye = to_float(add_lazy(add_lazy(add_lazy(mul_lazy(ck2::DC1, k1[s]), mul_lazy(ck2::DC3, k3[s])),
-                                                        add_lazy(mul_lazy(ck2::DC4, k4[s]), mul_lazy(ck2::DC5, k5[s]))),
-                                               mul_lazy(ck2::DC6, k6)));
-            if (sys.comp(tm, s) >= 0) {
-                if (isnan(ye) || isnan(yt[s].hi)) nan_flag = true;
-                err = fmaxf(err, __fdividef(fabsf(ye), fabsf(y[s].hi) + fabsf(k1[s].hi) + deltaf));
+        auto component = [&](int s, float ye, float ytn, float ys, float k1s) {
+            if (s < P && sys.comp(tm, s) >= 0) {
+                if (isnan(ye) || isnan(ytn)) nan_flag = true;
+                err = fmaxf(err, __fdividef(fabsf(ye), fabsf(ys) + fabsf(k1s) + deltaf));
             }
+        };
+#pragma unroll(P <= 64 ? P : 4)
+        for (int q = 0; q < NP; ++q) {
+            const F2x2 k6 = both(f, q) * F2x2(hh);
+            const F2x2 incr = add_lazy(add_lazy(mulc(ck2::C1, k1[q]), mulc(ck2::C3, k3[q])),
+                                       add_lazy(mulc(ck2::C4, k4[q]), mulc(ck2::C6, k6)));
+            yt[q] = y[q] + incr;
+            const F2x2 yd = add_lazy(add_lazy(add_lazy(mulc(ck2::DC1, k1[q]), mulc(ck2::DC3, k3[q])),
+                                              add_lazy(mulc(ck2::DC4, k4[q]), mulc(ck2::DC5, k5[q]))),
+                                     mulc(ck2::DC6, k6));
+            const f32x2 ye = add2(yd.hi, yd.lo);
+            component(q, half0(ye), half0(yt[q].hi), half0(y[q].hi), half0(k1[q].hi));
+            component(q + NP, half1(ye), half1(yt[q].hi), half1(y[q].hi), half1(k1[q].hi));
         }
         err = tm.max(err) * inv_rtolf;
         nan_flag = tm.any(nan_flag);
@@ -923,9 +1010,10 @@ struct RkckF2 {
             h = fmaxf(1.0e-20f, fminf(hmax, h * fac));
         bool bad = false;
 #pragma unroll(P <= 64 ? P : 4)
-        for (int s = 0; s < P; ++s) {
-            y[s] = yt[s];
-            if (sys.comp(tm, s) >= 0 && !isfinite(yt[s].hi)) bad = true;
+        for (int q = 0; q < NP; ++q) {
+            y[q] = yt[q];
+            if (sys.comp(tm, q) >= 0 && !isfinite(half0(yt[q].hi))) bad = true;
+            if (q + NP < P && sys.comp(tm, q + NP) >= 0 && !isfinite(half1(yt[q].hi))) bad = true;
         }
         if (tm.any(bad)) {
             status = ODE_ST_NONFINITE;
@@ -939,7 +1027,7 @@ struct RkckF2 {
 #pragma unroll(P <= 64 ? P : 4)
         for (int s = 0; s < P; ++s) {
             const int c = sys.comp(tm, s);
-            if (c >= 0) a.y_out[a.yidx_out(i, c)] = to_double(y[s]);
+            if (c >= 0) a.y_out[a.yidx_out(i, c)] = to_double(s < NP ? y[s % NP].first() : y[s % NP].second());
             if (a.carry != nullptr && c >= 0) a.carry[a.cidx(i, kCarryFixed + c)] = 0.0;
         }
         if (a.carry != nullptr && tm.lane == 0) {

@@ -18,6 +18,7 @@
 #include <sys/stat.h>
 #include <unistd.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -140,6 +141,69 @@ std::string lit(double x) {
     return "(" + s + ")";
 }
 
+// The two-float right-hand side on the packed instructions: species s and
+// s + NP (NP = (S + 1) / 2, the integrator's packs) accumulate together.  A
+// species' terms keep their order (each sum is the one the scalar code
+// forms, bit for bit); a term waits until its partner species has one too,
+// or is added by itself when the next one comes, so that few reactions'
+// rates stay live.  The 13-species network: 83 sums of eight instructions
+// become about 26 packed and 31 single ones; 1M systems in cost order
+// 121.3 -> 118.7 ms.
+std::string packed_rhs(const MassActionNet& net) {
+    const int S = net.n_species, NP = (S + 1) / 2;
+    std::ostringstream o;
+    struct Term {
+        int j;
+        bool plus;
+    };
+    std::vector<std::vector<Term>> wait(S);
+    std::vector<int> seen(S, 0);
+    auto rate = [](const Term& t) { return std::string(t.plus ? "r" : "-r") + std::to_string(t.j); };
+    auto single = [&](int s) {
+        o << "        a" << s << " = bode::add_lazy(a" << s << ", " << rate(wait[s].front()) << ");\n";
+        wait[s].erase(wait[s].begin());
+    };
+    auto pair = [&](int s, int m) {
+        o << "        { const bode::F2x2 t = bode::add_lazy(bode::F2x2(a" << s << ", a" << m << "), bode::F2x2("
+          << rate(wait[s].front()) << ", " << rate(wait[m].front()) << ")); a" << s << " = t.first(); a" << m
+          << " = t.second(); }\n";
+        wait[s].erase(wait[s].begin());
+        wait[m].erase(wait[m].begin());
+    };
+    auto add = [&](int s, Term t) {
+        if (!seen[s]) {
+            o << "        a" << s << " = " << rate(t) << ";\n";
+            seen[s] = 1;
+            return;
+        }
+        wait[s].push_back(t);
+        const int m = s < NP ? s + NP : s - NP;
+        if (m < S && !wait[m].empty())
+            pair(std::min(s, m), std::max(s, m));
+        else if (m >= S || wait[s].size() > 1)
+            single(s);
+    };
+    for (int s = 0; s < S; ++s) o << "        bode::F2 a" << s << "(0.0f, 0.0f);\n";
+    for (int j = 0; j < net.n_reactions; ++j) {
+        o << "        bode::F2 r" << j << " = k[" << j << "];";
+        for (int q = 0; q < net.n_reac[j]; ++q)
+            o << " r" << j << " = bode::mul_lazy(r" << j << ", y[" << (int)net.reac[j][q] << "]);";
+        o << "\n";
+        for (int q = 0; q < net.n_reac[j]; ++q) add(net.reac[j][q], {j, false});
+        for (int q = 0; q < net.n_prod[j]; ++q) add(net.prod[j][q], {j, true});
+    }
+    for (int s = 0; s < S; ++s)
+        while (!wait[s].empty()) single(s);
+    for (int q = 0; q < NP; ++q) {
+        if (q + NP < S)
+            o << "        { const bode::F2x2 t = bode::normalize(bode::F2x2(a" << q << ", a" << q + NP << ")); f[" << q
+              << "] = t.first(); f[" << q + NP << "] = t.second(); }\n";
+        else
+            o << "        f[" << q << "] = bode::normalize(a" << q << ");\n";
+    }
+    return o.str();
+}
+
 // The network as a Model (see rhs.cuh for the interface): rate constants in
 // registers, f written as straight-line code whose per-species accumulation
 // order is the reaction order (reactants, then products).
@@ -194,6 +258,9 @@ std::string model_source(const RhsEntry& r) {
     // the values an accumulator started at zero takes); the products and
     // sums go through the lazy two-float forms (the plain operations for
     // float and double), normalised once per species at the end
+    o << "      if constexpr (bode::is_f2<R>::value) {\n"
+      << packed_rhs(net) << "        return;\n"
+      << "      } else {\n";
     std::vector<int> seen(S, 0);
     for (int s = 0; s < S; ++s) o << "      R a" << s << ";\n";
     for (int j = 0; j < NR; ++j) {
@@ -220,7 +287,8 @@ std::string model_source(const RhsEntry& r) {
     for (int s = 0; s < S; ++s)
         if (!seen[s]) o << "      a" << s << " = R(0);\n";
     for (int s = 0; s < S; ++s) o << "      f[" << s << "] = bode::acc_value(a" << s << ");\n";
-    o << "    }\n";
+    o << "      }\n"
+      << "    }\n";
     // Gershgorin bound, row by row: J_sl accumulates reaction by reaction
     // -dr_j/dC_l per reactant occurrence of s, +dr_j/dC_l per product
     // occurrence, dr_j/dC_l summed over the reactant occurrences of l; the

@@ -166,6 +166,7 @@ extern "C" int rkc_integrate_noalloc(int32_t handle, int64_t nsys, const double*
     a.tend = tend;
     a.rtol = rtol;
     a.atol = atol;
+    a.u = UniformScalars(t0, tend, rtol, atol);
     a.n_accept = d_cnt[0];
     a.n_reject = d_cnt[1];
     a.n_rhs = d_cnt[2];

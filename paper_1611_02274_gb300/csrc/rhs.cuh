@@ -112,7 +112,56 @@ struct ChainModel {
                     }
             return acc;
         }
+        __device__ void neighbours(const Team<W>& tm, const R* y, int q, R& left, R& right) const {
+            left = tm.from_left(y[2 * q]);
+            right = tm.from_right(y[2 * q]);
+            if (q > 0) {
+                const R w = tm.bcast(y[q > 0 ? 2 * q - 2 : 0], W - 1);
+                if (tm.lane == 0) left = w;
+            }
+            if (q < G - 1) {
+                const R w = tm.bcast(y[q < G - 1 ? 2 * q + 2 : 0], 0);
+                if (tm.lane == W - 1) right = w;
+            }
+        }
+        // (xl - x) + (xr - x) of the neighbours that exist; a difference is
+        // normalised, so the first one needs no sum with zero
+        __device__ R coupling(const Team<W>& tm, const R* y, int q) const {
+            const int g = q * W + tm.lane;
+            R xl, xr;
+            neighbours(tm, y, q, xl, xr);
+            const F2x2 d = F2x2(xl, xr) - F2x2(y[2 * q]);
+            const R both = d.first() + d.second();
+            const bool left = g > 0, right = g + 1 < npts;
+            return left ? (right ? both : d.first()) : (right ? d.second() : R(0));
+        }
+        // two-float form on the packed instructions, the same operations in
+        // the same order; an even number of points a lane: two side by side
+        __device__ void rhs_packed(const Team<W>& tm, const R* y, R* f) const {
+            if constexpr (G == 1) {
+                const R x = y[0], v = y[1];
+                const F2x2 sq = F2x2(x, c) * F2x2(x, coupling(tm, y, 0));
+                f[0] = v;
+                f[1] = mu * (R(1) - sq.first()) * v - x + sq.second();
+            } else {
+#pragma unroll
+                for (int q = 0; q < G / 2; ++q) {
+                    const int q2 = q + G / 2;
+                    const F2x2 x(y[2 * q], y[2 * q2]), v(y[2 * q + 1], y[2 * q2 + 1]);
+                    const F2x2 cp = F2x2(c) * F2x2(coupling(tm, y, q), coupling(tm, y, q2));
+                    const F2x2 r = F2x2(mu) * (F2x2(R(1)) - x * x) * v - x + cp;
+                    f[2 * q] = y[2 * q + 1];
+                    f[2 * q2] = y[2 * q2 + 1];
+                    f[2 * q + 1] = r.first();
+                    f[2 * q2 + 1] = r.second();
+                }
+            }
+        }
         __device__ void rhs(const Team<W>& tm, R, const R* y, R* f) const {
+            if constexpr (is_f2<R>::value && (G == 1 || G % 2 == 0)) {
+                rhs_packed(tm, y, f);
+                return;
+            }
 #pragma unroll(G <= 32 ? G : 2)
             for (int q = 0; q < G; ++q) {
                 const int g = q * W + tm.lane;
@@ -203,7 +252,64 @@ struct BrussModel {
                     }
             return acc;
         }
+        // neighbours of grid point q of this lane in field `fld`, the ghosts at the ends
+        __device__ void neighbours(const Team<W>& tm, const R* y, int q, int fld, R bc, R& left, R& right) const {
+            const int g = q * W + tm.lane;
+            left = tm.from_left(y[2 * q + fld]);
+            right = tm.from_right(y[2 * q + fld]);
+            if (q > 0) {
+                const R w = tm.bcast(y[q > 0 ? 2 * q - 2 + fld : 0], W - 1);
+                if (tm.lane == 0) left = w;
+            }
+            if (q < G - 1) {
+                const R w = tm.bcast(y[q < G - 1 ? 2 * q + 2 + fld : 0], 0);
+                if (tm.lane == W - 1) right = w;
+            }
+            if (g == 0) left = bc;
+            if (g + 1 >= npts) right = bc;
+        }
+        // two-float form on the packed instructions, the same operations in
+        // the same order: with one point a lane, u and v side by side; with
+        // an even number, two points side by side (the integrator's packs)
+        __device__ void rhs_packed(const Team<W>& tm, const R* y, R* f) const {
+            const F2x2 Dp(D);
+            if constexpr (G == 1) {
+                R ul, ur, vl, vr;
+                neighbours(tm, y, 0, 0, ubc, ul, ur);
+                neighbours(tm, y, 0, 1, vbc, vl, vr);
+                const F2x2 p(y[0], y[1]);
+                const F2x2 diff = Dp * ((F2x2(ul, vl) - twice(p)) + F2x2(ur, vr));
+                const R uuv = y[0] * y[0] * y[1];
+                const F2x2 bu = F2x2(B1, B) * F2x2(y[0]);
+                const F2x2 t = F2x2(A, bu.second()) + F2x2(uuv, -uuv);
+                const F2x2 r = F2x2(t.first() - bu.first(), t.second()) + diff;
+                f[0] = r.first();
+                f[1] = r.second();
+            } else {
+#pragma unroll
+                for (int q = 0; q < G / 2; ++q) {
+                    const int q2 = q + G / 2;
+                    R l0, r0, l1, r1;
+                    const F2x2 u(y[2 * q], y[2 * q2]), v(y[2 * q + 1], y[2 * q2 + 1]);
+                    const F2x2 uuv = u * u * v;
+                    neighbours(tm, y, q, 0, ubc, l0, r0);
+                    neighbours(tm, y, q2, 0, ubc, l1, r1);
+                    const F2x2 fu = F2x2(A) + uuv - F2x2(B1) * u + Dp * (F2x2(l0, l1) - twice(u) + F2x2(r0, r1));
+                    neighbours(tm, y, q, 1, vbc, l0, r0);
+                    neighbours(tm, y, q2, 1, vbc, l1, r1);
+                    const F2x2 fv = F2x2(B) * u - uuv + Dp * (F2x2(l0, l1) - twice(v) + F2x2(r0, r1));
+                    f[2 * q] = fu.first();
+                    f[2 * q2] = fu.second();
+                    f[2 * q + 1] = fv.first();
+                    f[2 * q2 + 1] = fv.second();
+                }
+            }
+        }
         __device__ void rhs(const Team<W>& tm, R, const R* y, R* f) const {
+            if constexpr (is_f2<R>::value && (G == 1 || G % 2 == 0)) {
+                rhs_packed(tm, y, f);
+                return;
+            }
 #pragma unroll(G <= 32 ? G : 2)
             for (int q = 0; q < G; ++q) {
                 const int g = q * W + tm.lane;
