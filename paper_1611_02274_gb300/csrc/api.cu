@@ -335,6 +335,7 @@ std::map<std::tuple<int32_t, int, int, int, int, int>, std::pair<int, int>> g_ma
 void default_mapping(LaunchCfg* cfg, int block_req) {
     cfg->mapping = ODE_MAP_THREAD;
     cfg->block = block_req ? block_req : 128;
+    cfg->any_block = !block_req;
 }
 
 int tune_mapping(Workspace* ws, int32_t handle, const RhsEntry& rhs, int meth, int prec, bool use_jit, int block_req,
@@ -346,6 +347,7 @@ int tune_mapping(Workspace* ws, int32_t handle, const RhsEntry& rhs, int meth, i
     if (it != g_map_tuned.end()) {
         cfg->mapping = it->second.first;
         cfg->block = it->second.second;
+        cfg->any_block = false;
         return ODE_OK;
     }
     default_mapping(cfg, block_req);
@@ -375,6 +377,7 @@ int tune_mapping(Workspace* ws, int32_t handle, const RhsEntry& rhs, int meth, i
         if (cudaMalloc(&ws->tune_y, bytes) != cudaSuccess) return ODE_OK;  // untuned
         ws->tune_bytes = bytes;
     }
+    cfg->any_block = false;
     BatchArgs t = a;
     t.nsys = std::min<int64_t>(probe, sample_max);
     t.ld_in = a.nsys;
@@ -572,6 +575,7 @@ int integrate(Method method, int32_t handle, int64_t nsys, const double* y0, con
     cfg.team = 0;
     cfg.sm_count = ws->sm_count;
     cfg.stream = stream;
+    cfg.any_block = opts.mapping == ODE_MAP_THREAD && !opts.block_size;
     if (rhs.kind == ODE_RHS_KINETICS && opts.specrad != ODE_SPECRAD_POWER)
         return fail(ODE_ERR_UNSUPPORTED, "kinetics right-hand sides take the power method only (no Jacobian bound)");
     const int meth = method == kRkck ? kMethodRkck : kMethodRkc;
@@ -738,6 +742,7 @@ int ode_mapping_info(int32_t rhs_handle, int32_t method, int32_t precision, int3
         cfg.block = t->second.second;
     } else {
         default_mapping(&cfg, block_size);
+        if (cfg.any_block && precision == ODE_PREC_FP64) cfg.block = 32;
     }
     if (use_jit && cfg.block > jit_max_block(precision)) cfg.block = jit_max_block(precision);  // what launches
     *mapping = cfg.mapping;

@@ -722,7 +722,8 @@ int jit_launch(const RhsEntry& r, int method, int prec, const BatchArgs& a, cons
     NoCtx ctx;
     BatchArgs args = a;
     void* params[] = {&args, &ctx};
-    const int block = c.block > jit_max_block(prec) ? jit_max_block(prec) : c.block;
+    const int block = c.any_block && c.mapping == ODE_MAP_THREAD && prec == ODE_PREC_FP64 ? 32  // as in launch_method
+                      : c.block > jit_max_block(prec) ? jit_max_block(prec) : c.block;
     // the generated model is one thread per system with PER = species count
     const size_t smem = sizeof(float) * (size_t)k.smem_floats * (size_t)block;
     const int64_t threads = a.nsys;  // one thread per system

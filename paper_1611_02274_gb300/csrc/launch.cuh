@@ -29,12 +29,30 @@ struct LaunchCfg {
     int team;        // requested lanes per system (0 = family default; 32 keeps grids at a warp per system)
     int sm_count;
     cudaStream_t stream;
+    // the block size is neither the caller's nor timed: a one-launch kernel of
+    // the plain form then takes a warp per block.  Its warps share nothing,
+    // the FP64 pipe is what they wait for, a warp alone on its SM issues an
+    // FP64 instruction every 64 cycles where four take 76 each, and four-warp
+    // blocks leave a batch of a few warps per SM unevenly spread.  Measured,
+    // 128 / 32 threads: kinetics, 1,000 systems 94.9 / 83.2 ms; 32-point
+    // grids, 2,500 systems 26.0 / 18.6; van der Pol, 30,000 systems 7.04 /
+    // 6.11; 8,192 grids and 16,384 n-body systems the same.
+    bool any_block = false;
+};
+
+template <class T>
+struct is_double {
+    static constexpr bool value = false;
+};
+template <>
+struct is_double<double> {
+    static constexpr bool value = true;
 };
 
 template <class Method, class Ctx>
 cudaError_t launch_method(const BatchArgs& a, const Ctx& ctx, const LaunchCfg& c) {
     constexpr int W = Method::W;
-    const int block = c.block;
+    const int block = c.any_block && c.mapping == ODE_MAP_THREAD && is_double<typename Method::R>::value ? 32 : c.block;
     const size_t smem = sizeof(float) * Method::SMEM_FLOATS * (size_t)block;
     const int64_t threads = a.nsys * W;
     if (smem > 48 * 1024) {  // above the default dynamic shared-memory limit: opt in
@@ -74,8 +92,9 @@ enum { kMethodRkck = 0, kMethodRkc = 1 };
 // four sub-partitions times a step's FP64 work, in units of one point's:
 // G points a lane plus kOwn + kSum npts for the system (from the FP64
 // instruction counts of an RKC step: 150 a point, 110 a system and two per
-// point in the norm).  Measured on 32 points, wide / narrow: 8,192 systems
-// 68.3 / 52.5 ms.
+// point in the norm).  Measured on 32 points: 8,192 systems 68.3 ms wide,
+// 52.5 narrow; 608 systems wide 6.3 ms, where a round of the narrow kernel
+// takes 15.4.
 inline int grid_team_f64(int npts, int64_t nsys, int sm_count) {
     constexpr double kOwn = 0.75, kSum = 0.0133;
     int w = 1;

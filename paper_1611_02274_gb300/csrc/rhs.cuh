@@ -70,6 +70,39 @@ struct VdpModel {
     };
 };
 
+// The same system on two lanes, one component each: a step's element-wise
+// work takes half as many FP64 instructions per warp, at twice the warps.
+// For batches of the plain form that leave sub-partitions idle, where a
+// system's time is the number of FP64 instructions its warp issues.
+struct VdpPairModel {
+    static constexpr int W = 2, PER = 1;
+    using Ctx = NoCtx;
+    template <class R>
+    struct Sys {
+        R mu;
+        __device__ void load(const Ctx&, const Team<W>&, double param, int) { mu = (R)param; }
+        __device__ int comp(const Team<W>& tm, int) const { return tm.lane; }
+        template <class T>
+        __device__ T ordered_sum(const Team<W>& tm, const T* x) const {
+            T acc = T(0);
+            acc = acc + tm.bcast(x[0], 0);
+            acc = acc + tm.bcast(x[0], 1);
+            return acc;
+        }
+        __device__ void rhs(const Team<W>& tm, R, const R* y, R* f) const {
+            const R x = tm.bcast(y[0], 0), v = tm.bcast(y[0], 1);
+            const R dv = mu * (R(1) - x * x) * v - x;
+            f[0] = tm.lane == 0 ? v : dv;
+        }
+        __device__ R gershgorin(const Team<W>& tm, const R* y) const {
+            const R x = tm.bcast(y[0], 0), v = tm.bcast(y[0], 1);
+            const R j10 = mu * (R(-2) * x) * v - R(1);
+            const R j11 = mu * (R(1) - x * x);
+            return rmax(R(1), rabs(j10) + rabs(j11));
+        }
+    };
+};
+
 struct GridCtx {
     double A, B, ubc, vbc;  // Brusselator constants
     double coupling;        // chain coupling
