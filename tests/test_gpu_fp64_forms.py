@@ -73,3 +73,30 @@ def test_grid_shapes(family, method, points, nsys):
                        rng.uniform(-2.0, 2.0, (2 * points, nsys)), 10.0 ** rng.uniform(-1.0, 1.0, (1, nsys)), 0.0, 0.2,
                        1e-6, 1e-9)
     assert_same(w, method)
+
+
+@pytest.mark.parametrize("nsys", [1, 33, 9728, 9729])
+@pytest.mark.parametrize("method", ["rkck", "rkc"])
+def test_vdp_lanes(nsys, method):
+    """Two lanes a system up to a warp per sub-partition (152 SMs: 9728 systems), one past that."""
+    w = W.vdp(nsys=nsys, seed=nsys)
+    w.tend = 0.5
+    assert_same(w, method)
+
+
+@pytest.mark.parametrize("species,reactions", [(1, 1), (2, 3), (3, 5), (8, 12), (13, 27), (16, 32)])
+def test_network_sizes_two_float(species, reactions):
+    """Generated two-float networks of odd and even species counts: the packs' unused half, species without a term."""
+    import torch
+    net = W.make_network(11, species, reactions)
+    rng = np.random.default_rng(species)
+    n = 65
+    y0 = rng.uniform(0.1, 1.0, (species, n))
+    w = W.Workload("network", W.RHS_MASSACTION, W.METHOD_RKC, n, species, np.ascontiguousarray(y0 / y0.sum(axis=0)),
+                   rng.uniform(1000.0, 2000.0, (1, n)), 0.0, 1e-6, 1e-6, 1e-12, network=net)
+    h = B.register_workload(w)
+    y = B.integrate("rkc", h, torch.from_numpy(w.y0).cuda(), torch.from_numpy(w.params).cuda(), w.t0, w.tend, w.rtol,
+                    w.atol, precision=B.ODE_PREC_F2_LEAN, sync=True).cpu().numpy()
+    B.release(h)
+    r = O.integrate(O.model_for(w), W.METHOD_RKC, w.y0, w.params, w.t0, w.tend, w.rtol, w.atol)
+    assert (np.abs(y - r.y) / (np.abs(r.y) + w.atol)).max() <= 1e-5  # the two-float form's bar against the FP64 method
