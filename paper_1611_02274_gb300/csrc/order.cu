@@ -33,9 +33,14 @@ constexpr int kScanThreads = 1024;
 constexpr int kBinsPerThread = kOrderBins / kScanThreads;
 static_assert(kOrderBins % kScanThreads == 0, "bins split evenly over the scan block");
 
-// a cost as float: float32 estimates, or int32 counts (e.g. n_rhs)
+// a cost as float: float32 estimates, int32 counts (e.g. n_rhs), or an
+// FP64 parameter
 __device__ __forceinline__ float cost_at(const void* cost, int kind, int64_t i) {
-    return kind == 1 ? (float)static_cast<const int32_t*>(cost)[i] : static_cast<const float*>(cost)[i];
+    switch (kind) {
+    case kCostInt: return (float)static_cast<const int32_t*>(cost)[i];
+    case kCostParam: return (float)static_cast<const double*>(cost)[i];
+    default: return static_cast<const float*>(cost)[i];
+    }
 }
 
 // range[0] = lo, range[1] = hi (bit patterns of the positive costs)

@@ -100,3 +100,35 @@ def test_network_sizes_two_float(species, reactions):
     B.release(h)
     r = O.integrate(O.model_for(w), W.METHOD_RKC, w.y0, w.params, w.t0, w.tend, w.rtol, w.atol)
     assert (np.abs(y - r.y) / (np.abs(r.y) + w.atol)).max() <= 1e-5  # the two-float form's bar against the FP64 method
+
+
+@pytest.mark.parametrize("family,nsys", [("mass", 40003), ("mass", 19457), ("bruss", 5003), ("vdp", 100001), ("nbody", 9777)])
+def test_parameter_order(family, nsys):
+    """Batches that the library takes in parameter order (and n-body, which it does not): same results."""
+    w = {"mass": lambda: W.massaction(nsys=nsys, seed=5, tend=2e-7), "bruss": lambda: W.bruss(nsys=nsys, n=32, seed=5),
+         "vdp": lambda: W.vdp(nsys=nsys, seed=5), "nbody": lambda: W.pleiades(nsys=nsys, seed=5, tend=0.01)}[family]()
+    if family in ("bruss", "vdp"):
+        w.tend = 0.05
+    assert_same(w, "rkck" if w.method == W.METHOD_RKCK else "rkc")
+
+
+def test_two_float_order():
+    """The two-float network kernel: the order changes no bit."""
+    import torch
+    w = W.massaction(nsys=70001, seed=6, tend=5e-7)
+    h = B.register_workload(w)
+    y0, p = torch.from_numpy(w.y0).cuda(), torch.from_numpy(w.params).cuda()
+    out = []
+    for cost in (None, torch.ones(w.nsys, dtype=torch.float32, device="cuda")):
+        cnt = B.counters_like(w.nsys, "cuda")
+        y = B.integrate("rkc", h, y0, p, w.t0, w.tend, w.rtol, w.atol, precision=B.ODE_PREC_F2_LEAN, counters=cnt,
+                        cost=cost, mapping=B.ODE_MAP_THREAD, sync=True)
+        out.append((y.cpu().numpy(), cnt.n_rhs.cpu().numpy()))
+    # 3,000 of the systems as a batch of their own, in their own order
+    m = 3000
+    y = B.integrate("rkc", h, y0[:, :m].contiguous(), p[:, :m].contiguous(), w.t0, w.tend, w.rtol, w.atol,
+                    precision=B.ODE_PREC_F2_LEAN, sync=True).cpu().numpy()
+    B.release(h)
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
+    np.testing.assert_array_equal(out[0][0][:, :m], y)
