@@ -232,41 +232,44 @@ struct RkckF64 {
         }
         err = xm::div_by(err, rtol, rrtol);
         nan_flag = tm.any(nan_flag) || xm::is_nan(err);
+        // one power, one product and one way to the next attempt for the
+        // lanes of a warp that accept and those that reject
         const bool reject = nan_flag || xm::lt_nn(1.0, err);
-        const double fac = xm::pow_series(err, reject ? kPshrnk : kPgrow);
+        const double hs = kSafety * h * xm::pow_series(err, reject ? kPshrnk : kPgrow);
+        bool end = false;
         if (reject) {
             n_rej += 1;
-            if (nan_flag)
-                h = h * kP1;
-            else
-                h = xm::max_nn(kSafety * h * fac, kP1 * h);
-            if (h < 1.0e-20 || t + h == t) {
+            const double hp = kP1 * h;
+            h = nan_flag ? hp : xm::max_nn(hs, hp);
+            if (xm::lt_nn(h, 1.0e-20) || lost_in(t, h)) {
                 status = ODE_ST_H_UNDERFLOW;
-                stage = 0;
-                return;
+                end = true;
             }
-            loop_top();
-            return;
-        }
-        n_acc += 1;
-        t = t + h;
-        if (xm::lt_nn(kErrcon, err))
-            h = kSafety * h * fac;
-        else
-            h = h * 5.0;
-        h = xm::max_nn(1.0e-20, xm::min_nn(hmax, h));
-        bool bad = false;
+        } else {
+            n_acc += 1;
+            t = t + h;
+            h = xm::lt_nn(kErrcon, err) ? hs : h * 5.0;
+            h = xm::max_nn(1.0e-20, xm::min_nn(hmax, h));
+            bool bad = false;
 #pragma unroll(P <= 64 ? P : 4)
-        for (int s = 0; s < P; ++s) {
-            y[s] = yt[s];
-            if (sys.comp(tm, s) >= 0 && !xm::is_finite(yt[s])) bad = true;
+            for (int s = 0; s < P; ++s) {
+                y[s] = yt[s];
+                if (sys.comp(tm, s) >= 0 && !xm::is_finite(yt[s])) bad = true;
+            }
+            if (tm.any(bad)) {
+                status = ODE_ST_NONFINITE;
+                end = true;
+            }
         }
-        if (tm.any(bad)) {
-            status = ODE_ST_NONFINITE;
+        if (end)
             stage = 0;
-            return;
-        }
-        loop_top();
+        else
+            loop_top();
+    }
+    // t + h == t, asked of the exponents first
+    __device__ static bool lost_in(double t, double h) {
+        const int et = (__double2hiint(t) >> 20) & 0x7ff, eh = (__double2hiint(h) >> 20) & 0x7ff;
+        return et - eh >= 52 && t + h == t;
     }
 
     __device__ void store(const BatchArgs& a, const TM& tm, int64_t i) const {

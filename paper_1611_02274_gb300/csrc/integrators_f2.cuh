@@ -975,12 +975,14 @@ struct RkckF2 {
         }
         err = tm.max(err) * inv_rtolf;
         nan_flag = tm.any(nan_flag);
-        if (err > 1.0f || isnan(err) || nan_flag) {
+        // one power and one way to the next attempt for the lanes of a warp
+        // that accept and those that reject
+        const bool nan_err = isnan(err) || nan_flag, reject = err > 1.0f || nan_err;
+        const float fac = (float)kSafety * fpow(err, reject ? (float)kPshrnk : (float)kPgrow);
+        bool end = false;
+        if (reject) {
             n_rej += 1;
-            if (isnan(err) || nan_flag)
-                h = h * (HT)kP1;
-            else
-                h = h * (HT)fmaxf((float)kSafety * fpow(err, (float)kPshrnk), (float)kP1);
+            h = h * (nan_err ? (HT)kP1 : (HT)fmaxf(fac, (float)kP1));
             bool underflow;
             if constexpr (BK64)
                 underflow = h < 1.0e-20 || t + h == t;
@@ -988,39 +990,39 @@ struct RkckF2 {
                 underflow = h < 1.0e-20f || h <= tabsf * 2.2e-16f;
             if (underflow) {
                 status = ODE_ST_H_UNDERFLOW;
-                stage = 0;
-                return;
+                end = true;
             }
-            loop_top();
-            return;
-        }
-        n_acc += 1;
-        if constexpr (BK64) {
-            t = t + h;
-        } else if (h >= remf * 0.999999f) {
-            remf = reml = 0.0f;  // the step covered what was left
         } else {
-            df_sub(remf, reml, h);
-            tabsf = fabsf(tendf - remf);
-        }
-        const float fac = (err > (float)kErrcon) ? (float)kSafety * fpow(err, (float)kPgrow) : 5.0f;
-        if constexpr (BK64)
-            h = fmax(1.0e-20, fmin(hmax, h * (double)fac));
-        else
-            h = fmaxf(1.0e-20f, fminf(hmax, h * fac));
-        bool bad = false;
+            n_acc += 1;
+            if constexpr (BK64) {
+                t = t + h;
+            } else if (h >= remf * 0.999999f) {
+                remf = reml = 0.0f;  // the step covered what was left
+            } else {
+                df_sub(remf, reml, h);
+                tabsf = fabsf(tendf - remf);
+            }
+            const float grow = (err > (float)kErrcon) ? fac : 5.0f;
+            if constexpr (BK64)
+                h = fmax(1.0e-20, fmin(hmax, h * (double)grow));
+            else
+                h = fmaxf(1.0e-20f, fminf(hmax, h * grow));
+            bool bad = false;
 #pragma unroll(P <= 64 ? P : 4)
-        for (int q = 0; q < NP; ++q) {
-            y[q] = yt[q];
-            if (sys.comp(tm, q) >= 0 && !isfinite(half0(yt[q].hi))) bad = true;
-            if (q + NP < P && sys.comp(tm, q + NP) >= 0 && !isfinite(half1(yt[q].hi))) bad = true;
+            for (int q = 0; q < NP; ++q) {
+                y[q] = yt[q];
+                if (sys.comp(tm, q) >= 0 && !isfinite(half0(yt[q].hi))) bad = true;
+                if (q + NP < P && sys.comp(tm, q + NP) >= 0 && !isfinite(half1(yt[q].hi))) bad = true;
+            }
+            if (tm.any(bad)) {
+                status = ODE_ST_NONFINITE;
+                end = true;
+            }
         }
-        if (tm.any(bad)) {
-            status = ODE_ST_NONFINITE;
+        if (end)
             stage = 0;
-            return;
-        }
-        loop_top();
+        else
+            loop_top();
     }
 
     __device__ void store(const BatchArgs& a, const TM& tm, int64_t i) const {
