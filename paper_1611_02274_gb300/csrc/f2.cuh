@@ -231,11 +231,11 @@ template <class T>
 __device__ __forceinline__ T acc_value(T a) { return normalize(a); }
 
 // Per-system constants of a right-hand side (e.g. rate constants): an
-// array in registers for the plain and FP32 forms; for the two-float forms,
-// whose pairs would take twice the registers, a row of the block's shared
-// memory that the integrator binds (SMEM_FLOATS floats per thread, an odd
-// number of pairs so that a half-warp's 8-byte loads fall in distinct
-// banks).
+// array in registers for the FP32 forms; for the two-float and the plain
+// forms, whose pairs and doubles would take twice the registers, a row of the
+// block's shared memory that the integrator binds (SMEM_FLOATS floats per
+// thread, an odd number of pairs so that a half-warp's 8-byte loads fall in
+// distinct banks).
 template <class R, int N>
 struct ConstStore {
     static constexpr int SMEM_FLOATS = 0;
@@ -244,14 +244,18 @@ struct ConstStore {
     __device__ const R& operator[](int j) const { return v[j]; }
     __device__ void bind(float*) {}
 };
-template <int N>
-struct ConstStore<F2, N> {
+template <class R, int N>
+struct SmemConsts {
     static constexpr int SMEM_FLOATS = 2 * (N | 1);
-    F2* v;
-    __device__ F2& operator[](int j) { return v[j]; }
-    __device__ const F2& operator[](int j) const { return v[j]; }
-    __device__ void bind(float* row) { v = reinterpret_cast<F2*>(row); }
+    R* v;
+    __device__ R& operator[](int j) { return v[j]; }
+    __device__ const R& operator[](int j) const { return v[j]; }
+    __device__ void bind(float* row) { v = reinterpret_cast<R*>(row); }
 };
+template <int N>
+struct ConstStore<F2, N> : SmemConsts<F2, N> {};
+template <int N>
+struct ConstStore<double, N> : SmemConsts<double, N> {};
 
 // warp shuffles of a pair (both words from the same lane)
 __device__ __forceinline__ F2 shfl_xor(unsigned m, F2 v, int o, int w) {

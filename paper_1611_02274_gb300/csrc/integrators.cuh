@@ -44,6 +44,17 @@ struct ModelSmem<M, void_t_<decltype(M::SMEM_FLOATS)>> {
     static constexpr int value = M::SMEM_FLOATS;
 };
 
+// Floats of shared memory per thread a system asks for to hold its
+// constants (Sys::CONST_SMEM, 0 if it declares none).
+template <class S, class = void>
+struct ConstSmem {
+    static constexpr int value = 0;
+};
+template <class S>
+struct ConstSmem<S, void_t_<decltype(S::CONST_SMEM)>> {
+    static constexpr int value = S::CONST_SMEM;
+};
+
 // PH_PROPOSE: waiting for the warp's evaluation of the proposal network
 // (two-float RKC with an in-kernel network, mlp_warp.cuh)
 enum : int { PH_DONE = 0, PH_F0, PH_SR, PH_TRIAL, PH_STAGE, PH_FINAL, PH_PROPOSE };
@@ -96,9 +107,11 @@ __device__ __forceinline__ void carry_scalars(const BatchArgs& a, int64_t i, boo
 template <class Model>
 struct RkckF64 {
     static constexpr bool kStepSync = false;  // fixed six stages: lanes stay aligned
-    static constexpr int SMEM_FLOATS = ModelSmem<Model>::value;
+    static constexpr int C_SMEM = ConstSmem<typename Model::template Sys<double>>::value;
+    static constexpr int SMEM_FLOATS = C_SMEM + ModelSmem<Model>::value;
     __device__ void bind_smem(float* base, int stride) {
-        if constexpr (SMEM_FLOATS > 0) sys.bind(base, stride);
+        if constexpr (C_SMEM > 0) sys.bind_consts(base + threadIdx.x * C_SMEM);
+        if constexpr (ModelSmem<Model>::value > 0) sys.bind(base + C_SMEM * stride, stride);
     }
     static constexpr int W = Model::W, P = Model::PER;
     using R = double;
@@ -296,15 +309,30 @@ struct RkckF64 {
 template <class Model>
 struct RkcF64 {
     static constexpr bool kStepSync = true;  // variable stage count: hold at the step end
-    static constexpr int SMEM_FLOATS = ModelSmem<Model>::value;
-    __device__ void bind_smem(float* base, int stride) {
-        if constexpr (SMEM_FLOATS > 0) sys.bind(base, stride);
-    }
     static constexpr int W = Model::W, P = Model::PER;
+    // The power method's vector, touched every 25 steps, and a generated
+    // network's rate constants live in shared-memory rows (an odd number of
+    // doubles per thread) where a thread holds a whole system: in registers
+    // they spilled the integrator's state, 1,530 -> 312 bytes in the
+    // 13-species kernel; 100,003 systems in parameter order 238 -> 214 ms.
+    static constexpr int V_SMEM = W == 1 && P >= 8 && P <= 32 ? 2 * (P | 1) : 0;
+    static constexpr int C_SMEM = ConstSmem<typename Model::template Sys<double>>::value;
+    static constexpr int SMEM_FLOATS = V_SMEM + C_SMEM + ModelSmem<Model>::value;
+    __device__ void bind_smem(float* base, int stride) {
+        if constexpr (V_SMEM > 0) v.bind(base + threadIdx.x * V_SMEM);
+        if constexpr (C_SMEM > 0) sys.bind_consts(base + V_SMEM * stride + threadIdx.x * C_SMEM);
+        if constexpr (ModelSmem<Model>::value > 0) sys.bind(base + (V_SMEM + C_SMEM) * stride, stride);
+    }
+    struct RegRow {
+        double a[P];
+        __device__ double& operator[](int s) { return a[s]; }
+        __device__ const double& operator[](int s) const { return a[s]; }
+    };
     using R = double;
     using TM = Team<W>;
     typename Model::template Sys<double> sys;
-    double yn[P], Fn[P], v[P], w1[P], w2[P];  // w1 = w_{j-1}, w2 = w_{j-2}
+    typename Pick<(V_SMEM > 0), SmemConsts<double, P>, RegRow>::type v;
+    double yn[P], Fn[P], w1[P], w2[P];  // w1 = w_{j-1}, w2 = w_{j-2}
     double t, tend, rtol, atol, hmax, hmin, h, h_old, err_old, sigma;
     double lerr_old, rn;                        // log err_old; 1 / n (xm::div_by)
     double dynrm, sig;                          // power method in progress
@@ -371,7 +399,8 @@ struct RkcF64 {
     __device__ bool in_stages() const { return phase == PH_STAGE; }
     __device__ bool at_step_end() const { return phase == PH_FINAL; }
 
-    __device__ double sumsq(const TM& tm, const double* x) const {
+    template <class Row>
+    __device__ double sumsq(const TM& tm, const Row& x) const {
         double sq[P];
 #pragma unroll(P <= 64 ? P : 4)
         for (int s = 0; s < P; ++s) sq[s] = x[s] * x[s];

@@ -30,17 +30,6 @@ namespace bode {
 // sqrt(2.22e-16): the power method's relative perturbation (Appendix)
 constexpr float kSqrtUround = 1.4899664e-8f;
 
-// Floats of shared memory per thread a system asks for to hold its
-// constants (Sys::CONST_SMEM, 0 if it declares none).
-template <class S, class = void>
-struct ConstSmem {
-    static constexpr int value = 0;
-};
-template <class S>
-struct ConstSmem<S, void_t_<decltype(S::CONST_SMEM)>> {
-    static constexpr int value = S::CONST_SMEM;
-};
-
 // Systems whose constants may come precomputed (Sys::kPreConsts, load_pre).
 template <class S, class = void>
 struct PreConsts {
