@@ -127,13 +127,16 @@ __device__ __forceinline__ float loss_grad(int o, float p, float t, float* loss)
 // deep, and added 5,300 terms per block with atomics.  Rows of the tiles are
 // kRow floats long, so that the rows a warp reads at once start in different
 // banks.  The whole call on
-// 262,144 rows, 2 epochs of 64 batches: 22.0 -> 4.7 ms.
+// 262,144 rows, 2 epochs of 64 batches: 22.0 -> 3.96 ms, of which the host's
+// two shuffles take about 1.5.
 constexpr int kTile = 32;
 constexpr int kTrainThreads = 256;
 constexpr int kRow = kH + 4;
 constexpr int kXRow = 52;  // inputs padded to 16, 32 or 48 columns
+// floats of a block's row of sums: the parameters, the loss, whole 16-byte words
+__host__ __device__ constexpr int part_stride(int n_in) { return (mlp_nparams(n_in) + 1 + 3) / 4 * 4; }
 struct TrainSmem {
-    float w1t[kMlpMaxIn * kRow];  // W1 by input
+    float w1t[(kMlpMaxIn + 3) / 4 * 4 * kRow];  // W1 by input, zero rows up to a multiple of 4
     float w2[kH * kRow];          // W2 by output neuron
     float w2t[kH * kRow];         // W2 by input neuron
     float w3[kMlpOut * kH];
@@ -148,21 +151,26 @@ __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast
 __device__ __forceinline__ void st4(float* p, const float* v) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
-// acc[r][c] += w[c] * v over a run of K inputs: w rows are kRow long and hold
-// four outputs at `col`, the two samples' inputs are rows v0 and v1
+// acc[r][c] += w[c] * v over a run of K inputs (K a multiple of 4): w rows are
+// kRow long and hold four outputs, the two samples' inputs are rows v0 and v1
 __device__ __forceinline__ void mac_inputs(const float* w, const float* v0, const float* v1, int K, float (&acc)[2][4]) {
 #pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-        const float4 q = ld4(w + k * kRow);
-        const float a = v0[k], b = v1[k];
-        acc[0][0] = fmaf(q.x, a, acc[0][0]);
-        acc[0][1] = fmaf(q.y, a, acc[0][1]);
-        acc[0][2] = fmaf(q.z, a, acc[0][2]);
-        acc[0][3] = fmaf(q.w, a, acc[0][3]);
-        acc[1][0] = fmaf(q.x, b, acc[1][0]);
-        acc[1][1] = fmaf(q.y, b, acc[1][1]);
-        acc[1][2] = fmaf(q.z, b, acc[1][2]);
-        acc[1][3] = fmaf(q.w, b, acc[1][3]);
+    for (int k = 0; k < K; k += 4) {
+        const float4 a4 = ld4(v0 + k), b4 = ld4(v1 + k);
+        const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 q = ld4(w + (k + i) * kRow);
+            const float a = av[i], b = bv[i];
+            acc[0][0] = fmaf(q.x, a, acc[0][0]);
+            acc[0][1] = fmaf(q.y, a, acc[0][1]);
+            acc[0][2] = fmaf(q.z, a, acc[0][2]);
+            acc[0][3] = fmaf(q.w, a, acc[0][3]);
+            acc[1][0] = fmaf(q.x, b, acc[1][0]);
+            acc[1][1] = fmaf(q.y, b, acc[1][1]);
+            acc[1][2] = fmaf(q.z, b, acc[1][2]);
+            acc[1][3] = fmaf(q.w, b, acc[1][3]);
+        }
     }
 }
 
@@ -174,13 +182,43 @@ __global__ void __launch_bounds__(kTrainThreads) k_mlp_grad(const __nv_bfloat16*
     extern __shared__ __align__(16) unsigned char raw[];
     TrainSmem& sm = *reinterpret_cast<TrainSmem*>(raw);
     const int tid = threadIdx.x;
+    // Everything a block reads is asked for before anything is waited for:
+    // the chain row index -> inputs is the only one that is two reads long.
+    // Eight threads a row: the row's inputs, and its targets on three of them.
+    const int rs = tid >> 3, rl = tid & 7;
+    auto row_of = [&](int64_t t) -> int64_t {
+        const int64_t q = t * kTile + rs;
+        return q < n ? (perm ? (int64_t)perm[q] : q) : -1;
+    };
+    const int64_t row0 = row_of(blockIdx.x);
     // weights (BF16 -> FP32)
-    for (int e = tid; e < kH * n_in; e += kTrainThreads)
-        sm.w1t[(e % n_in) * kRow + e / n_in] = __bfloat162float(w16[mlp_w1(n_in) + e]);
-    for (int q = tid; q < kH * kH / 8; q += kTrainThreads) {  // lanes take consecutive rows: no bank conflicts
-        const int j = q & (kH - 1), k = (q / kH) * 8;
-        const uint4 u = *reinterpret_cast<const uint4*>(w16 + mlp_w2(n_in) + j * kH + k);  // 128-byte rows
-        const uint32_t word[4] = {u.x, u.y, u.z, u.w};
+    constexpr int kW1 = (kH * kMlpMaxIn + kTrainThreads - 1) / kTrainThreads, kW2 = kH * kH / 8 / kTrainThreads;
+    __nv_bfloat16 v1[kW1], v3[2], vb[2];
+    uint4 v2[kW2];
+#pragma unroll
+    for (int i = 0; i < kW2; ++i) {  // lanes take consecutive rows (128 bytes): no bank conflicts in shared memory
+        const int q = tid + i * kTrainThreads, j = q & (kH - 1), k = (q / kH) * 8;
+        v2[i] = *reinterpret_cast<const uint4*>(w16 + mlp_w2(n_in) + j * kH + k);
+    }
+#pragma unroll
+    for (int i = 0; i < kW1; ++i)
+        if (tid + i * kTrainThreads < kH * n_in) v1[i] = w16[mlp_w1(n_in) + tid + i * kTrainThreads];
+    if (tid < kMlpOut * kH) v3[0] = w16[mlp_w3(n_in) + tid];
+    if (tid < kMlpOut) v3[1] = w16[mlp_b3(n_in) + tid];
+    if (tid < kH) {
+        vb[0] = w16[mlp_b1(n_in) + tid];
+        vb[1] = w16[mlp_b2(n_in) + tid];
+    }
+#pragma unroll
+    for (int i = 0; i < kW1; ++i) {
+        const int e = tid + i * kTrainThreads;
+        if (e < kH * n_in) sm.w1t[(e % n_in) * kRow + e / n_in] = __bfloat162float(v1[i]);
+    }
+    for (int e = n_in * kRow + tid; e < (n_in + 3) / 4 * 4 * kRow; e += kTrainThreads) sm.w1t[e] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < kW2; ++q) {
+        const int j = (tid + q * kTrainThreads) & (kH - 1), k = ((tid + q * kTrainThreads) / kH) * 8;
+        const uint32_t word[4] = {v2[q].x, v2[q].y, v2[q].z, v2[q].w};
         float v[8];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -192,37 +230,40 @@ __global__ void __launch_bounds__(kTrainThreads) k_mlp_grad(const __nv_bfloat16*
 #pragma unroll
         for (int i = 0; i < 8; ++i) sm.w2t[(k + i) * kRow + j] = v[i];
     }
-    if (tid < kMlpOut * kH) sm.w3[tid] = __bfloat162float(w16[mlp_w3(n_in) + tid]);
+    if (tid < kMlpOut * kH) sm.w3[tid] = __bfloat162float(v3[0]);
+    if (tid < kMlpOut) sm.b3[tid] = __bfloat162float(v3[1]);
     if (tid < kH) {
-        sm.b1[tid] = __bfloat162float(w16[mlp_b1(n_in) + tid]);
-        sm.b2[tid] = __bfloat162float(w16[mlp_b2(n_in) + tid]);
+        sm.b1[tid] = __bfloat162float(vb[0]);
+        sm.b2[tid] = __bfloat162float(vb[1]);
     }
-    if (tid < kMlpOut) sm.b3[tid] = __bfloat162float(w16[mlp_b3(n_in) + tid]);
 
     const int jg = 4 * (tid & 15), s0 = 2 * (tid >> 4);     // layer products: 4 neurons x 2 samples
-    const int jt = 4 * (tid & 15), kt = 4 * (tid >> 4);     // W2 gradient: 4 x 4 elements
+    const int jt = 4 * (tid >> 4), kt = 4 * (tid & 15);     // W2 gradient: 4 x 4 elements, rows along the lanes
     const int jr = tid & 63, role = tid >> 6;               // W1 gradient: a neuron, a quarter of the inputs
     const int kper = 4 * ((n_in + 15) / 16);                // inputs per quarter: 4, 8 or 12
     float gW2[4][4] = {}, gW1[12] = {}, gB = 0.0f, gW3[kMlpOut] = {}, lsum = 0.0f;
     const int64_t tiles = (n + kTile - 1) / kTile;
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const int rows = (int)min((int64_t)kTile, n - t * kTile);
         // normalised inputs, zero past n_in and past the last row
-        for (int e = tid; e < kTile * 4 * kper; e += kTrainThreads) {
-            const int s = e / (4 * kper), k = e % (4 * kper);
-            float v = 0.0f;
-            if (s < rows && k < n_in) {
-                const int64_t q = t * kTile + s, r = perm ? perm[q] : q;
-                v = (X[r * n_in + k] - norm.x_mean[k]) / norm.x_scale[k];
-            }
-            sm.x[s * kXRow + k] = v;
+        const int64_t r = t == blockIdx.x ? row0 : row_of(t);
+        float xin[6], target = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) xin[i] = r >= 0 && rl + 8 * i < n_in ? X[r * n_in + rl + 8 * i] : 0.0f;
+        if (r >= 0 && rl < kMlpOut) target = Y[r * kMlpOut + rl];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            const int k = rl + 8 * i;
+            if (k < 4 * kper)
+                sm.x[rs * kXRow + k] = r >= 0 && k < n_in ? (xin[i] - norm.x_mean[k < kMlpMaxIn ? k : 0]) /
+                                                                norm.x_scale[k < kMlpMaxIn ? k : 0]
+                                                          : 0.0f;
         }
         __syncthreads();
         float z1[2][4], z2[2][4], out[4];
         {
             const float4 b = ld4(sm.b1 + jg);
             for (int r = 0; r < 2; ++r) z1[r][0] = b.x, z1[r][1] = b.y, z1[r][2] = b.z, z1[r][3] = b.w;
-            mac_inputs(sm.w1t + jg, sm.x + s0 * kXRow, sm.x + (s0 + 1) * kXRow, n_in, z1);
+            mac_inputs(sm.w1t + jg, sm.x + s0 * kXRow, sm.x + (s0 + 1) * kXRow, (n_in + 3) / 4 * 4, z1);
         }
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
@@ -244,7 +285,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_mlp_grad(const __nv_bfloat16*
         }
         __syncthreads();
         {  // outputs: eight lanes a sample, then the loss and its gradient
-            const int s = tid >> 3, l = tid & 7;
+            const int s = rs, l = rl;
             float z3[kMlpOut] = {};
 #pragma unroll
             for (int i = 0; i < kH / 8; ++i) {
@@ -257,11 +298,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_mlp_grad(const __nv_bfloat16*
                 for (int d = 4; d > 0; d >>= 1) z3[o] += __shfl_xor_sync(0xffffffffu, z3[o], d);
                 if (l == o) {
                     float g = 0.0f;
-                    if (s < rows) {
-                        const int64_t q = t * kTile + s, r = perm ? perm[q] : q;
-                        const float y = (Y[r * kMlpOut + o] - norm.y_mean[o]) / norm.y_scale[o];
-                        g = loss_grad(o, z3[o] + sm.b3[o], y, &lsum);
-                    }
+                    if (r >= 0) g = loss_grad(o, z3[o] + sm.b3[o], (target - norm.y_mean[o]) / norm.y_scale[o], &lsum);
                     sm.g3[s * 4 + o] = g;
                 }
             }
@@ -320,13 +357,17 @@ __global__ void __launch_bounds__(kTrainThreads) k_mlp_grad(const __nv_bfloat16*
         }
         __syncthreads();  // the tile is read before the next one is written
     }
-    float* p = part + (int64_t)blockIdx.x * (mlp_nparams(n_in) + 1);
+    // the block's row of sums, written in whole sectors: W2 as 16-byte words
+    // of consecutive lanes, W1 by way of shared memory (scattered 4-byte
+    // stores cost the kernel more than its products did)
+    float* p = part + (int64_t)blockIdx.x * part_stride(n_in);
+#pragma unroll
     for (int i = 0; i < 12; ++i)
-        if (i < kper && role * kper + i < n_in) p[mlp_w1(n_in) + jr * n_in + role * kper + i] = gW1[i];
+        if (i < kper && role * kper + i < n_in) sm.w1t[(role * kper + i) * kRow + jr] = gW1[i];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) p[mlp_w2(n_in) + (jt + r) * kH + kt + c] = gW2[r][c];
+    for (int r = 0; r < 4; ++r) st4(p + mlp_w2(n_in) + (jt + r) * kH + kt, gW2[r]);
+    __syncthreads();
+    for (int e = tid; e < kH * n_in; e += kTrainThreads) p[mlp_w1(n_in) + e] = sm.w1t[(e % n_in) * kRow + e / n_in];
     if (role == 0) p[mlp_b1(n_in) + jr] = gB;
     if (role == 1) p[mlp_b2(n_in) + jr] = gB;
     if (role == 2)
@@ -348,16 +389,21 @@ __global__ void __launch_bounds__(kTrainThreads) k_mlp_grad(const __nv_bfloat16*
 // master and its BF16 copy and adds to *loss; otherwise the mean gradient to
 // out and the summed loss to *loss.
 template <bool ADAM>
-__global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, int blocks, int np, float n_rows,
+__global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, int blocks, int stride, int np, float n_rows,
                                                 float* __restrict__ out, float* master, __nv_bfloat16* w16, float* m,
                                                 float* v, float lr, float b1, float b2, float eps, float c1, float c2,
                                                 float* loss) {
     __shared__ float sums[8][32];
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
-    float s = 0.0f;
+    float s = 0.0f, m0 = 0.0f, v0 = 0.0f, w0 = 0.0f;
+    if (ADAM && slice == 0 && k < np) {  // asked for before the sums are waited for
+        m0 = m[k];
+        v0 = v[k];
+        w0 = master[k];
+    }
     if (k <= np)
-#pragma unroll 8
-        for (int b = slice; b < blocks; b += 8) s += part[(int64_t)b * (np + 1) + k];
+#pragma unroll 16
+        for (int b = slice; b < blocks; b += 8) s += part[(int64_t)b * stride + k];
     sums[slice][lane] = s;
     __syncthreads();
     if (slice || k > np) return;
@@ -371,11 +417,11 @@ __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, 
         return;
     }
     const float g = s * (1.0f / n_rows);
-    const float mk = b1 * m[k] + (1.0f - b1) * g;
-    const float vk = b2 * v[k] + (1.0f - b2) * g * g;
+    const float mk = b1 * m0 + (1.0f - b1) * g;
+    const float vk = b2 * v0 + (1.0f - b2) * g * g;
     m[k] = mk;
     v[k] = vk;
-    const float w = master[k] - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+    const float w = w0 - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
     master[k] = w;
     w16[k] = __float2bfloat16_rn(w);
 }
@@ -578,7 +624,7 @@ int grad_blocks(const Mlp& net, int64_t n) {
 
 // room for the block sums of gradients over up to n rows
 int reserve_part(Mlp& net, int64_t n) {
-    const size_t need = sizeof(float) * (size_t)grad_blocks(net, n) * (net.nparams + 1);
+    const size_t need = sizeof(float) * (size_t)grad_blocks(net, n) * part_stride(net.n_in);
     if (net.part_bytes >= need) return ODE_OK;
     cudaFree(net.part);
     net.part = nullptr;
@@ -749,7 +795,7 @@ int ode_mlp_gradient(int32_t handle, const float* X, const float* Y, int64_t n, 
     cudaError_t e = run_grad(*net, X, Y, nullptr, n, s);
     if (e != cudaSuccess) return cuda_fail(e, "gradient kernel");
     // mean over the rows
-    k_reduce<false><<<net->nparams / 32 + 1, 256, 0, s>>>(net->part, grad_blocks(*net, n), net->nparams, (float)n, grad_out,
+    k_reduce<false><<<net->nparams / 32 + 1, 256, 0, s>>>(net->part, grad_blocks(*net, n), part_stride(net->n_in), net->nparams, (float)n, grad_out,
                                                           nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 1, 1, net->loss);
     float l = 0;
     e = cudaGetLastError();
@@ -772,42 +818,40 @@ int ode_mlp_train(int32_t handle, const float* X, const float* Y, int64_t n, con
     if (!net->has_norm) return fail(ODE_ERR_ARG, "call ode_mlp_fit_normalization first");
     cudaStream_t s = (cudaStream_t)stream;
     if ((rc = reserve_part(*net, std::min<int64_t>(n, o->batch)))) return rc;
-    int32_t* perm = nullptr;
-    cudaError_t e = cudaMalloc(&perm, sizeof(int32_t) * n);
+    int32_t* perm = nullptr;  // the epoch's permutation, then the epochs' losses
+    cudaError_t e = cudaMalloc(&perm, sizeof(int32_t) * (size_t)(n + o->epochs));
     if (e != cudaSuccess) return fail(ODE_ERR_NOMEM, "permutation buffer");
+    float* losses = reinterpret_cast<float*>(perm + n);
     std::vector<int32_t> hp(n);
     std::mt19937_64 rng(o->seed);
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    for (int ep = 0; ep < o->epochs; ++ep) {
+    e = cudaMemsetAsync(losses, 0, sizeof(float) * o->epochs, s);
+    for (int ep = 0; ep < o->epochs && e == cudaSuccess; ++ep) {
+        // shuffled while the previous epoch's batches run
         for (int64_t k = 0; k < n; ++k) hp[k] = (int32_t)k;
         std::shuffle(hp.begin(), hp.end(), rng);
-        cudaMemcpyAsync(perm, hp.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s);
-        cudaMemsetAsync(net->loss, 0, sizeof(float), s);
-        for (int64_t b0 = 0; b0 < n; b0 += o->batch) {
+        e = cudaMemcpyAsync(perm, hp.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the copy has read hp
+        for (int64_t b0 = 0; b0 < n && e == cudaSuccess; b0 += o->batch) {
             const int64_t bn = std::min<int64_t>(o->batch, n - b0);
             e = run_grad(*net, X, Y, perm + b0, bn, s);
             net->step += 1;
             const float c1 = 1.0f - std::pow(b1, (float)net->step), c2 = 1.0f - std::pow(b2, (float)net->step);
-            if (e == cudaSuccess) {
-                k_reduce<true><<<net->nparams / 32 + 1, 256, 0, s>>>(net->part, grad_blocks(*net, bn), net->nparams, (float)bn,
-                                                                     nullptr, net->master, net->w16, net->m, net->v, o->lr,
-                                                                     b1, b2, eps, c1, c2, net->loss);
-                e = cudaGetLastError();
-            }
-            if (e != cudaSuccess) {
-                cudaFree(perm);
-                return cuda_fail(e, "training step");
-            }
+            if (e != cudaSuccess) break;
+            k_reduce<true><<<net->nparams / 32 + 1, 256, 0, s>>>(net->part, grad_blocks(*net, bn), part_stride(net->n_in), net->nparams, (float)bn,
+                                                                 nullptr, net->master, net->w16, net->m, net->v, o->lr, b1,
+                                                                 b2, eps, c1, c2, losses + ep);
+            e = cudaGetLastError();
         }
-        float l = 0;
-        e = cudaMemcpyAsync(&l, net->loss, sizeof(float), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) {
-            cudaFree(perm);
-            return cuda_fail(e, "training");
-        }
-        if (loss_history) loss_history[ep] = l / (float)n;
     }
+    std::vector<float> l(o->epochs);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(l.data(), losses, sizeof(float) * o->epochs, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        cudaFree(perm);
+        return cuda_fail(e, "training");
+    }
+    for (int ep = 0; loss_history && ep < o->epochs; ++ep) loss_history[ep] = l[ep] / (float)n;
     cudaFree(perm);
     return refresh_packed(*net, s);
 }
