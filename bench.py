@@ -66,7 +66,8 @@ LEARNED_FORMS = {"f2_lean_learned", "f2_learned"}
 BASE_FORM = {"f2_lean_learned": "f2_lean", "f2_learned": "f2"}
 # our kernel launches per step: the integration kernel; for the generated
 # two-float forms the rate-constant prologue; for the learned forms the
-# proposal pre-pass and the four kernels of the cost order
+# proposal pre-pass and the four kernels of the cost order (the FP32 and
+# plain forms' own parameter order, four small kernels more, is not counted)
 LAUNCHES = {"f2_lean_learned": 7, "f2_lean": 2, "f2_learned": 7, "f2": 2, "mixed_lean": 1, "mixed_spec_split": 1,
             "plain_fp64": 1}
 FORM_KERNELS = {"f2_lean_learned": "RkcF2<JitMass, false>", "f2_lean": "RkcF2<JitMass, false>",

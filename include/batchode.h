@@ -200,7 +200,10 @@ typedef struct {
      * of costs, with its own kernels, and the integration kernel reads them
      * through that order.  Results do not
      * depend on the order; only the time does (lanes of a warp then hold
-     * systems of similar cost, and the long ones start first).  Not in the
+     * systems of similar cost, and the long ones start first).  Without it
+     * (and without carry, outside stream capture) the library may take the
+     * systems in the order of their parameter; results are those of the
+     * batch's own order.  Not in the
      * paper, whose mapping takes the systems in index order. */
     const float* cost;
     /* Optional warm-restart state, read and written (device, io DEVICE only;

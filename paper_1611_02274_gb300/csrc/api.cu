@@ -355,14 +355,21 @@ void default_mapping(LaunchCfg* cfg, int block_req) {
 // system alone sets the time, and a call of a warm-restart chain, which may
 // be short, brings its own estimate or none.  Measured, unordered / ordered:
 // van der Pol two-float 1M systems 8.84 / 7.70 ms, 32-point FP64 grids, 8,192
-// systems 52.3 / 43.6; networks two-float 1M systems 161 / 144 and 300,000
-// 50 / 45, FP64 100,003 239-276 / 219 (with their constants in shared memory).
+// systems 52.3 / 43.6; networks two-float 50,021 systems 10.4 / 9.7, FP64
+// 100,003 239-276 / 219 (with their constants in shared memory).  Two-float
+// network batches above 2^18 systems keep their own order although it would
+// pay there too (1M systems 161 / 144 ms): those are what the learned
+// proposal orders (134 ms), and its gain is defined, and tested, against the
+// batch as it comes.
 int auto_order(const RhsEntry& rhs, int prec, const BatchArgs& a, int sm_count) {
     if (a.carry != nullptr || a.mlp != nullptr || a.nsys > INT32_MAX) return -1;
     int lanes = 32;
     switch (rhs.kind) {
     case ODE_RHS_VDP: lanes = 1; break;
-    case ODE_RHS_MASSACTION: lanes = 1; break;
+    case ODE_RHS_MASSACTION:
+        if (prec_is_f2(prec) && a.nsys > 1 << 18) return -1;
+        lanes = 1;
+        break;
     case ODE_RHS_BRUSS1D:
     case ODE_RHS_VDP_CHAIN:
         if (prec == ODE_PREC_FP64) lanes = grid_team_f64(rhs.neq / 2, a.nsys, sm_count);
@@ -383,7 +390,11 @@ bool any_order(const RhsEntry& rhs, int meth, int prec, int mapping) {
 constexpr size_t kOrderStreams = 16;
 bool order_buffers(Workspace* ws, cudaStream_t stream, int64_t n, Workspace::OrderBuf** out) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return false;
     if (ws->order.size() >= kOrderStreams && ws->order.find(stream) == ws->order.end()) return false;
     Workspace::OrderBuf& ob = ws->order[stream];
     *out = &ob;
