@@ -40,6 +40,12 @@ int bode_fma_peak(int fp64, int32_t iters, double* gflops, double* ms);
  * omega_i sums this product forms. */
 int bode_stoich_bench(int32_t rhs, int32_t variant, int64_t nsys, int32_t reps, double* ms, double* max_err);
 
+/* What the calling thread's last integration launch took: info[0] whether
+ * the systems were read through an order, info[1] lanes per system, info[2]
+ * threads per block, info[3] ODE_MAP_THREAD or ODE_MAP_QUEUE.  Returns 0, or
+ * ODE_ERR_ARG (info is NULL). */
+int bode_last_launch(int32_t* info);
+
 #ifdef __cplusplus
 }
 #endif

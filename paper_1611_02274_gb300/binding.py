@@ -34,7 +34,7 @@ EXPORTED = ["ode_rhs_register", "ode_rhs_release", "ode_rhs_prepare", "rkck_inte
             "ode_mlp_train", "ode_mlp_gradient", "ode_mlp_apply", "ode_mlp_apply_warp", "ode_mlp_propose", "ode_mlp_get_params",
             "ode_mlp_set_params", "ode_ragged_plan_create", "ode_ragged_plan_launch", "ode_ragged_plan_info",
             "ode_ragged_plan_destroy", "ode_tuning_reset", "ode_cost_order", "ode_cost_order_i32",
-            "ode_mapping_info"]
+            "ode_mapping_info", "bode_last_launch"]
 NOALLOC_SCRATCH_BYTES = 16 << 20
 
 
@@ -464,6 +464,13 @@ def mapping_info(handle: int, method: str, precision: int, codegen: int = ODE_CO
     if rc not in (ODE_OK, ODE_ERR_UNSUPPORTED):
         _check(rc)
     return int(m.value), int(b.value), rc == ODE_OK
+
+
+def last_launch() -> dict:
+    """bode_last_launch: order, lanes per system, block size and mapping of this thread's last launch."""
+    v = (C.c_int32 * 4)()
+    _check(load().bode_last_launch(v))
+    return {"ordered": bool(v[0]), "lanes": v[1], "block": v[2], "mapping": v[3]}
 
 
 def tuning_reset() -> None:

@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "batchode.h"
+#include "batchode_bench.h"
 #include "jit.h"
 #include "launch.cuh"
 #include "order.h"
@@ -51,19 +52,32 @@ int cuda_fail(cudaError_t e, const char* what) {
 // buffer for host-pointer calls.
 constexpr int kCursorRing = 1024;
 constexpr int kRkcTabMax = 256;  // stage counts with tabulated coefficients
+constexpr int kOrderBufs = 8;
+constexpr size_t kOrderBytes = 256u << 20;
 struct Workspace {
     unsigned long long* cursors = nullptr;  // kCursorRing + 1: the last one for tuning runs
     int next_cursor = 0;
     double* tune_y = nullptr;  // output of mapping-tuning runs, grow-only
     size_t tune_bytes = 0;
-    // cost-ordering buffers per stream (grow-only): calls on one stream run
-    // in order, calls on different streams get their own buffers
+    // buffers of the caller's cost order per stream (grow-only): calls on one
+    // stream run in order, calls on different streams get their own buffers.
+    // The automatic order never touches them: a graph captured from a call
+    // with a cost holds them, and calls without one did not use to.
     struct OrderBuf {
         int32_t* bins = nullptr;
         int32_t* index = nullptr;
         int64_t cap = 0;
     };
     std::map<cudaStream_t, OrderBuf> order;
+    // the automatic order's buffers (OrderScratch): at most kOrderBytes in all
+    struct AutoBuf {
+        int32_t* mem = nullptr;
+        size_t words = 0;
+        cudaEvent_t done = nullptr;  // behind the last launch that read it
+        uint64_t turn = 0;
+    };
+    AutoBuf auto_bufs[kOrderBufs];
+    uint64_t auto_turn = 0;
     // precomputed right-hand-side constants per stream (grow-only)
     struct ConstBuf {
         void* ptr = nullptr;
@@ -383,31 +397,93 @@ bool any_order(const RhsEntry& rhs, int meth, int prec, int mapping) {
     return !(joins && prec_is_f2(prec) && meth == kMethodRkc && mapping == ODE_MAP_QUEUE);
 }
 
-// A stream's order buffers for n systems, for an order the caller did not
-// ask for: false (the batch keeps its own order) on a capturing stream, whose
-// graph must not hold buffers that a larger call replaces, past kOrderStreams
-// streams, and when memory is out.
-constexpr size_t kOrderStreams = 16;
-bool order_buffers(Workspace* ws, cudaStream_t stream, int64_t n, Workspace::OrderBuf** out) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+// Memory of one call's automatic order, from the workspace's few buffers: a
+// call takes one that is idle (or makes its stream wait for one that is not),
+// and gives it back behind its launch with an event on its own stream.  What
+// orders two users of a buffer is that event, never a stream's handle
+// (cudaStreamPerThread is one handle for a stream per thread), and no captured
+// graph holds a buffer.  index stays NULL -- the batch keeps its own order --
+// on a capturing stream and when memory is out.  Called under g_mu.
+struct OrderScratch {
+    Workspace::AutoBuf* buf = nullptr;
+    int32_t* index = nullptr;
+    cudaStream_t stream = nullptr;
+    // event queries and allocations must not disturb a capture in another thread
+    struct Relaxed {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+        ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    };
+    int32_t* bins() const { return buf->mem; }
+    bool take(Workspace* ws, cudaStream_t s, int64_t n) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (cap != cudaStreamCaptureStatusNone) return false;
+        constexpr size_t kBins = (kOrderScratchWords + 63) / 64 * 64;  // words, whole 256-byte lines
+        const size_t words = kBins + (size_t)n;
+        Relaxed relaxed;
+        // the smallest idle buffer that is large enough, else room for a new
+        // one in the place of a smaller idle one, else the one used longest ago
+        Workspace::AutoBuf *fit = nullptr, *small = nullptr, *oldest = nullptr;
+        size_t held = 0;
+        for (Workspace::AutoBuf& b : ws->auto_bufs) {
+            held += b.words;
+            if (b.mem && cudaEventQuery(b.done) != cudaSuccess) {
+                cudaGetLastError();
+                if (b.words >= words && (!oldest || b.turn < oldest->turn)) oldest = &b;
+                continue;
+            }
+            if (b.words >= words) {
+                if (!fit || b.words < fit->words) fit = &b;
+            } else if (!small || b.words < small->words) {
+                small = &b;
+            }
+        }
+        if (!fit && small && sizeof(int32_t) * (held - small->words + words) <= kOrderBytes) {
+            Workspace::AutoBuf& b = *small;
+            cudaFree(b.mem);
+            b.mem = nullptr;
+            b.words = 0;
+            if ((b.done || cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming) == cudaSuccess) &&
+                cudaMalloc(&b.mem, sizeof(int32_t) * words) == cudaSuccess) {
+                b.words = words;
+                fit = &b;
+            } else {
+                b.mem = nullptr;
+                cudaGetLastError();  // not the caller's error: the batch keeps its order
+            }
+        }
+        if (!fit && oldest && cudaStreamWaitEvent(s, oldest->done, 0) == cudaSuccess) fit = oldest;
+        if (!fit) return false;
+        buf = fit;
+        buf->turn = ++ws->auto_turn;
+        index = buf->mem + kBins;
+        stream = s;
+        return true;
+    }
+    ~OrderScratch() {
+        if (!buf || cudaEventRecord(buf->done, stream) == cudaSuccess) return;
         cudaGetLastError();
-        return false;
+        cudaStreamSynchronize(stream);  // without its event the buffer is idle only once the stream is
     }
-    if (cap != cudaStreamCaptureStatusNone) return false;
-    if (ws->order.size() >= kOrderStreams && ws->order.find(stream) == ws->order.end()) return false;
-    Workspace::OrderBuf& ob = ws->order[stream];
-    *out = &ob;
-    if (ob.cap < n) {
-        cudaFree(ob.index);
-        ob.index = nullptr;
-        ob.cap = 0;
-        if (cudaMalloc(&ob.index, sizeof(int32_t) * (size_t)n) == cudaSuccess) ob.cap = n;
+    // gives idle buffers back
+    static void trim(Workspace& ws) {
+        Relaxed relaxed;
+        for (Workspace::AutoBuf& b : ws.auto_bufs) {
+            if (!b.mem) continue;
+            if (cudaEventQuery(b.done) != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            cudaFree(b.mem);
+            b.mem = nullptr;
+            b.words = 0;
+        }
     }
-    if (!ob.bins && cudaMalloc(&ob.bins, sizeof(int32_t) * kOrderScratchWords) != cudaSuccess) ob.bins = nullptr;
-    if (ob.cap < n || !ob.bins) cudaGetLastError();  // not the caller's error: the batch keeps its order
-    return ob.cap >= n && ob.bins;
-}
+};
 
 int tune_mapping(Workspace* ws, int32_t handle, const RhsEntry& rhs, int meth, int prec, bool use_jit, int block_req,
                  const BatchArgs& a, int order, LaunchCfg* cfg) {
@@ -487,14 +563,14 @@ int tune_mapping(Workspace* ws, int32_t handle, const RhsEntry& rhs, int meth, i
             t.nsys = std::min<int64_t>(sample_max, std::max<int64_t>(std::min<int64_t>(65536, sample_max), want));
         }
         t.index = nullptr;  // the sample in the order the batch will take
-        Workspace::OrderBuf* ob = nullptr;
-        if (order >= 0 && any_order(rhs, meth, prec, c.mapping) && order_buffers(ws, c.stream, t.nsys, &ob)) {
-            e = order_by_cost(t.params, order, t.nsys, ob->bins, ob->index, ws->sm_count, c.stream);
+        OrderScratch ob;
+        if (order >= 0 && any_order(rhs, meth, prec, c.mapping) && ob.take(ws, c.stream, t.nsys)) {
+            e = order_by_cost(t.params, order, t.nsys, ob.bins(), ob.index, ws->sm_count, c.stream);
             if (e != cudaSuccess) {
                 rc = cuda_fail(e, "mapping tuning");
                 break;
             }
-            t.index = ob->index;
+            t.index = ob.index;
         }
         e = cudaEventRecord(e0, c.stream);
         if (e == cudaSuccess) rc = dispatch(rhs, meth, prec, use_jit, t, c);
@@ -687,11 +763,11 @@ int integrate(Method method, int32_t handle, int64_t nsys, const double* y0, con
         rc = tune_mapping(ws, handle, rhs, meth, opts.precision, use_jit, opts.block_size, a, order, &cfg);
         if (rc) return rc;
     }
-    Workspace::OrderBuf* auto_buf = nullptr;
-    if (order >= 0 && any_order(rhs, meth, opts.precision, cfg.mapping) && order_buffers(ws, stream, nsys, &auto_buf)) {
-        e = order_by_cost(d_p, order, nsys, auto_buf->bins, auto_buf->index, ws->sm_count, stream);
+    OrderScratch auto_buf;  // given back behind the launch when this call returns
+    if (order >= 0 && any_order(rhs, meth, opts.precision, cfg.mapping) && auto_buf.take(ws, stream, nsys)) {
+        e = order_by_cost(d_p, order, nsys, auto_buf.bins(), auto_buf.index, ws->sm_count, stream);
         if (e != cudaSuccess) return cuda_fail(e, "cost ordering");
-        a.index = auto_buf->index;
+        a.index = auto_buf.index;
     }
     if (opts.cost) {
         Workspace::OrderBuf& ob = ws->order[stream];
@@ -774,6 +850,12 @@ int ode_rhs_release(int32_t rhs_handle) {
     if (it_r == g_reg.end()) return fail(ODE_ERR_HANDLE, "unknown rhs handle %d", rhs_handle);
     if (it_r->second.kin_alloc) cudaFree(it_r->second.kin_alloc);
     g_reg.erase(it_r);
+    if (g_reg.empty()) {  // the last right-hand side: the current device's idle order buffers go too
+        int dev = 0;
+        auto ws = cudaGetDevice(&dev) == cudaSuccess ? g_ws.find(dev) : g_ws.end();
+        if (ws != g_ws.end()) OrderScratch::trim(ws->second);
+        cudaGetLastError();
+    }
     for (auto it = g_map_tuned.begin(); it != g_map_tuned.end();)
         it = std::get<0>(it->first) == rhs_handle ? g_map_tuned.erase(it) : std::next(it);
     return ODE_OK;
@@ -883,6 +965,14 @@ int ode_tuning_reset(void) {
         g_map_tuned.clear();
     }
     ragged_tuning_reset();
+    return ODE_OK;
+}
+
+int bode_last_launch(int32_t* info) {
+    if (!info) return ODE_ERR_ARG;
+    const LaunchInfo& l = g_last_launch;
+    const int32_t v[4] = {l.ordered, l.lanes, l.block, l.mapping};
+    std::memcpy(info, v, sizeof(v));
     return ODE_OK;
 }
 

@@ -727,6 +727,7 @@ int jit_launch(const RhsEntry& r, int method, int prec, const BatchArgs& a, cons
     // the generated model is one thread per system with PER = species count
     const size_t smem = sizeof(float) * (size_t)k.smem_floats * (size_t)block;
     const int64_t threads = a.nsys;  // one thread per system
+    g_last_launch = LaunchInfo{a.index != nullptr, 1, block, c.mapping};
     cudaError_t e;
     if (smem > 48 * 1024) {  // above the default dynamic shared-memory limit: opt in
         e = cudaFuncSetAttribute((const void*)k.kstatic, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -40,6 +40,13 @@ struct LaunchCfg {
     bool any_block = false;
 };
 
+// What the calling thread's last launch took (bode_last_launch).
+struct LaunchInfo {
+    int32_t ordered = 0;  // systems read through an order or a plan's index
+    int32_t lanes = 0, block = 0, mapping = 0;
+};
+inline thread_local LaunchInfo g_last_launch;
+
 template <class T>
 struct is_double {
     static constexpr bool value = false;
@@ -55,6 +62,7 @@ cudaError_t launch_method(const BatchArgs& a, const Ctx& ctx, const LaunchCfg& c
     const int block = c.any_block && c.mapping == ODE_MAP_THREAD && is_double<typename Method::R>::value ? 32 : c.block;
     const size_t smem = sizeof(float) * Method::SMEM_FLOATS * (size_t)block;
     const int64_t threads = a.nsys * W;
+    g_last_launch = LaunchInfo{a.index != nullptr, W, block, c.mapping};
     if (smem > 48 * 1024) {  // above the default dynamic shared-memory limit: opt in
         cudaError_t e = cudaFuncSetAttribute(k_static<Method, Ctx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
