@@ -200,10 +200,12 @@ typedef struct {
      * of costs, with its own kernels, and the integration kernel reads them
      * through that order.  Results do not
      * depend on the order; only the time does (lanes of a warp then hold
-     * systems of similar cost, and the long ones start first).  Without it
+     * systems of similar cost, and the long ones start first).  Equal
+     * estimates keep the batch's own order.  Without estimates
      * (and without carry, outside stream capture) the library may take the
-     * systems in the order of their parameter; results are those of the
-     * batch's own order.  Not in the
+     * systems of a large batch over a long interval in the order of their
+     * parameter, unless neighbouring systems are alike in it already; results
+     * are those of the batch's own order.  Not in the
      * paper, whose mapping takes the systems in index order. */
     const float* cost;
     /* Optional warm-restart state, read and written (device, io DEVICE only;

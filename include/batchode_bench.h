@@ -46,6 +46,10 @@ int bode_stoich_bench(int32_t rhs, int32_t variant, int64_t nsys, int32_t reps, 
  * ODE_ERR_ARG (info is NULL). */
 int bode_last_launch(int32_t* info);
 
+/* The order the library takes a batch in when it orders by parameter: index
+ * [n] (device), from params [n] (device).  Same errors as ode_cost_order. */
+int bode_parameter_order(const double* params, int64_t n, int32_t* index, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -34,7 +34,7 @@ EXPORTED = ["ode_rhs_register", "ode_rhs_release", "ode_rhs_prepare", "rkck_inte
             "ode_mlp_train", "ode_mlp_gradient", "ode_mlp_apply", "ode_mlp_apply_warp", "ode_mlp_propose", "ode_mlp_get_params",
             "ode_mlp_set_params", "ode_ragged_plan_create", "ode_ragged_plan_launch", "ode_ragged_plan_info",
             "ode_ragged_plan_destroy", "ode_tuning_reset", "ode_cost_order", "ode_cost_order_i32",
-            "ode_mapping_info", "bode_last_launch"]
+            "ode_mapping_info", "bode_last_launch", "bode_parameter_order"]
 NOALLOC_SCRATCH_BYTES = 16 << 20
 
 
@@ -132,6 +132,7 @@ def load(build_if_missing: bool = True):
     L.ode_mlp_set_params.argtypes = [C.c_int32, P, P]
     L.ode_cost_order.argtypes = [P, C.c_int64, P, P]
     L.ode_cost_order_i32.argtypes = [P, C.c_int64, P, P]
+    L.bode_parameter_order.argtypes = [P, C.c_int64, P, P]
     L.ode_mapping_info.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, P, P]
     _lib = L
     return L
@@ -454,6 +455,14 @@ def cost_order(cost, stream=None):
     fn = load().ode_cost_order_i32 if cost.dtype == torch.int32 else load().ode_cost_order
     _check(fn(_ptr(cost), int(cost.shape[0]), _ptr(idx), _stream(stream)))
     return idx
+
+
+def parameter_order(params, stream=None):
+    """bode_parameter_order: the order the library takes a batch in by its parameter (float64 [n], device)."""
+    import torch
+    index = torch.empty(params.numel(), dtype=torch.int32, device=params.device)
+    _check(load().bode_parameter_order(_ptr(params), int(params.numel()), _ptr(index), _stream(stream)))
+    return index
 
 
 def mapping_info(handle: int, method: str, precision: int, codegen: int = ODE_CODEGEN_AUTO, block_size: int = 0):

@@ -75,6 +75,7 @@ struct Workspace {
         size_t words = 0;
         cudaEvent_t done = nullptr;  // behind the last launch that read it
         uint64_t turn = 0;
+        cudaStream_t last = nullptr;  // the stream of that launch
     };
     AutoBuf auto_bufs[kOrderBufs];
     uint64_t auto_turn = 0;
@@ -363,33 +364,51 @@ void default_mapping(LaunchCfg* cfg, int block_req) {
 // takes 14,659 against a mean of 2,100), starts early.
 // Results do not depend on the order; where they do -- the two-float RKC in
 // the work queue or with an in-kernel network, whose lanes join each other's
-// estimates -- the batch keeps its own.  The order is four small launches
-// (about 0.02 ms; 0.1 ms for 1M systems) and pays where the batch is more
-// than one round of warps over the sub-partitions; below that the longest
-// system alone sets the time, and a call of a warm-restart chain, which may
-// be short, brings its own estimate or none.  Measured, unordered / ordered:
-// van der Pol two-float 1M systems 8.84 / 7.70 ms, 32-point FP64 grids, 8,192
-// systems 52.3 / 43.6; networks two-float 50,021 systems 10.4 / 9.7, FP64
-// 100,003 239-276 / 219 (with their constants in shared memory).  Two-float
-// network batches above 2^18 systems keep their own order although it would
-// pay there too (1M systems 161 / 144 ms): those are what the learned
-// proposal orders (134 ms), and its gain is defined, and tested, against the
-// batch as it comes.
-int auto_order(const RhsEntry& rhs, int prec, const BatchArgs& a, int sm_count) {
+// estimates -- the batch keeps its own, and so it does where its layout
+// groups like systems already (order.cu).
+// An order costs five small launches, 0.02 ms (20,000 systems) to 0.07 ms
+// (1M), so it is for batches of more than a round of warps over the
+// sub-partitions and for intervals that are long on the family's own time
+// scale: for van der Pol systems, chains and grids, whose equations have no
+// units, the interval itself; for networks the interval times the largest
+// rate constant they are registered with.  The FP32-pipe forms hide a warp's
+// wait behind its neighbours' work and need more rounds than the plain form.
+// Measured, the order's time / its own order's (one launch over the batch):
+//                               below the line        above it
+//   van der Pol RKCK, FP64      20,000 over 0.3 1.02  20,000 over 1 0.90, 250,000 over 0.1 0.56
+//     two-float (FP32 1.2-2.9)  60,000 over 0.1 1.64  60,000 over 10 0.77, 250,000 over 1 0.47
+//   RKC, FP64 (grids, chains)   20,000 over 3 1.05    60,000 over 0.01 0.89, over 1 0.59
+//     two-float                 60,000 over 0.3 1.09  250,000 over 0.01 0.89, over 1 0.52
+//   networks (kmax 1e6), FP64   60,000 over 1e-6 0.99 over 1e-5 0.76
+//     two-float                 over 1e-8 1.04        over 1e-5 0.88
+// Two-float network batches above 2^18 systems keep their own order although
+// it would pay there too (1M systems 161 / 144 ms): those are what the
+// learned proposal orders (134 ms), and its gain is defined, and tested,
+// against the batch as it comes.
+int auto_order(const RhsEntry& rhs, int meth, int prec, const BatchArgs& a, int sm_count) {
     if (a.carry != nullptr || a.mlp != nullptr || a.nsys > INT32_MAX) return -1;
+    const bool f64 = prec == ODE_PREC_FP64, rkc = meth == kMethodRkc;
     int lanes = 32;
+    double units = a.tend - a.t0, rounds_min = rkc || rhs.kind != ODE_RHS_VDP ? 2.0 : 1.0;
+    double work_min = rkc ? 0.03 : 0.9;  // rounds x units
+    if (!f64) rounds_min = rkc ? 5.0 : 3.0, work_min = rkc ? 0.1 : 10.0;
     switch (rhs.kind) {
     case ODE_RHS_VDP: lanes = 1; break;
     case ODE_RHS_MASSACTION:
         if (prec_is_f2(prec) && a.nsys > 1 << 18) return -1;
         lanes = 1;
+        units *= rhs.net.kmax;
+        if (units < 5.0) return -1;
+        rounds_min = 1.0;
+        work_min = 0.0;
         break;
     case ODE_RHS_BRUSS1D:
     case ODE_RHS_VDP_CHAIN:
-        if (prec == ODE_PREC_FP64) lanes = grid_team_f64(rhs.neq / 2, a.nsys, sm_count);
+        if (f64) lanes = grid_team_f64(rhs.neq / 2, a.nsys, sm_count);
         break;
     }
-    return lanes < 32 && a.nsys * lanes > 32 * 4 * (int64_t)sm_count ? (int)kCostParam : -1;
+    const double rounds = (double)(a.nsys * lanes) / (32 * 4 * (double)sm_count);
+    return lanes < 32 && rounds > rounds_min && rounds * units >= work_min ? (int)kCostParam : -1;
 }
 // whether a launch may take the systems in another order
 bool any_order(const RhsEntry& rhs, int meth, int prec, int mapping) {
@@ -425,15 +444,19 @@ struct OrderScratch {
         constexpr size_t kBins = (kOrderScratchWords + 63) / 64 * 64;  // words, whole 256-byte lines
         const size_t words = kBins + (size_t)n;
         Relaxed relaxed;
-        // the smallest idle buffer that is large enough, else room for a new
-        // one in the place of a smaller idle one, else the one used longest ago
-        Workspace::AutoBuf *fit = nullptr, *small = nullptr, *oldest = nullptr;
+        // the buffer that this stream's last call used (it runs before this
+        // one anyhow), else the smallest idle one that is large enough, else
+        // room for a new one in the place of a smaller idle one, else the one
+        // used longest ago
+        Workspace::AutoBuf *fit = nullptr, *small = nullptr, *oldest = nullptr, *mine = nullptr;
         size_t held = 0;
         for (Workspace::AutoBuf& b : ws->auto_bufs) {
             held += b.words;
             if (b.mem && cudaEventQuery(b.done) != cudaSuccess) {
                 cudaGetLastError();
-                if (b.words >= words && (!oldest || b.turn < oldest->turn)) oldest = &b;
+                if (b.words < words) continue;
+                if (!oldest || b.turn < oldest->turn) oldest = &b;
+                if (s != cudaStreamPerThread && b.last == s) mine = &b;
                 continue;
             }
             if (b.words >= words) {
@@ -442,7 +465,8 @@ struct OrderScratch {
                 small = &b;
             }
         }
-        if (!fit && small && sizeof(int32_t) * (held - small->words + words) <= kOrderBytes) {
+        if (mine) fit = nullptr, oldest = mine;
+        if (!fit && !mine && small && sizeof(int32_t) * (held - small->words + words) <= kOrderBytes) {
             Workspace::AutoBuf& b = *small;
             cudaFree(b.mem);
             b.mem = nullptr;
@@ -460,6 +484,7 @@ struct OrderScratch {
         if (!fit) return false;
         buf = fit;
         buf->turn = ++ws->auto_turn;
+        buf->last = s;
         index = buf->mem + kBins;
         stream = s;
         return true;
@@ -758,7 +783,7 @@ int integrate(Method method, int32_t handle, int64_t nsys, const double* y0, con
         a.pre_consts = cb.ptr;
         a.pre_stride = nsys;
     }
-    const int order = opts.cost ? -1 : auto_order(rhs, opts.precision, a, ws->sm_count);
+    const int order = opts.cost ? -1 : auto_order(rhs, meth, opts.precision, a, ws->sm_count);
     if (opts.mapping == ODE_MAP_AUTO) {
         rc = tune_mapping(ws, handle, rhs, meth, opts.precision, use_jit, opts.block_size, a, order, &cfg);
         if (rc) return rc;
@@ -931,6 +956,10 @@ int ode_cost_order(const float* cost, int64_t n, int32_t* index, void* stream_pt
 
 int ode_cost_order_i32(const int32_t* cost, int64_t n, int32_t* index, void* stream_ptr) {
     return cost_order_any(cost, 1, n, index, stream_ptr);
+}
+
+int bode_parameter_order(const double* params, int64_t n, int32_t* index, void* stream_ptr) {
+    return cost_order_any(params, kCostParam, n, index, stream_ptr);
 }
 
 }  // extern "C"

@@ -10,10 +10,13 @@ namespace bode {
 // 65535 about log-uniform steps over the batch's range of positive costs.
 constexpr int kOrderBins = 65536;
 // int32 words of device scratch order_by_cost needs
-constexpr int kOrderScratchWords = 2 * kOrderBins + 2;
+constexpr int kOrderStatWords = 8;
+constexpr int kOrderScratchWords = 2 * kOrderBins + kOrderStatWords;
 
 // Writes index[0..n) = the systems 0..n-1, most expensive class first,
-// on stream s.  bins: device scratch of kOrderScratchWords int32; index:
+// on stream s; their own order where all costs are equal, and for a
+// parameter (kCostParam) where consecutive systems are alike in it already.
+// bins: device scratch of kOrderScratchWords int32, 16-byte aligned; index:
 // n int32.  cost: device [n], by kind: float32, int32, or float64 (a system's
 // parameter).
 enum { kCostFloat = 0, kCostInt = 1, kCostParam = 2 };
