@@ -404,7 +404,7 @@ int auto_order(const RhsEntry& rhs, int meth, int prec, const BatchArgs& a, int 
         break;
     case ODE_RHS_BRUSS1D:
     case ODE_RHS_VDP_CHAIN:
-        if (f64) lanes = grid_team_f64(rhs.neq / 2, a.nsys, sm_count);
+        if (f64) lanes = grid_team_f64(rhs.neq / 2, a.nsys, sm_count, rhs.kind == ODE_RHS_VDP_CHAIN, meth, true);
         break;
     }
     const double rounds = (double)(a.nsys * lanes) / (32 * 4 * (double)sm_count);

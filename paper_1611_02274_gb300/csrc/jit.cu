@@ -722,7 +722,9 @@ int jit_launch(const RhsEntry& r, int method, int prec, const BatchArgs& a, cons
     NoCtx ctx;
     BatchArgs args = a;
     void* params[] = {&args, &ctx};
-    const int block = c.any_block && c.mapping == ODE_MAP_THREAD && prec == ODE_PREC_FP64 ? 32  // as in launch_method
+    const bool warp_block = c.any_block && c.mapping == ODE_MAP_THREAD && prec == ODE_PREC_FP64 &&
+                            a.nsys <= kWarpBlocksPerSm * 32 * (int64_t)c.sm_count;  // as in launch_method
+    const int block = warp_block ? 32
                       : c.block > jit_max_block(prec) ? jit_max_block(prec) : c.block;
     // the generated model is one thread per system with PER = species count
     const size_t smem = sizeof(float) * (size_t)k.smem_floats * (size_t)block;

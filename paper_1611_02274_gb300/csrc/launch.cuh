@@ -36,9 +36,13 @@ struct LaunchCfg {
     // blocks leave a batch of a few warps per SM unevenly spread.  Measured,
     // 128 / 32 threads: kinetics, 1,000 systems 94.9 / 83.2 ms; 32-point
     // grids, 2,500 systems 26.0 / 18.6; van der Pol, 30,000 systems 7.04 /
-    // 6.11; 8,192 grids and 16,384 n-body systems the same.
+    // 6.11; 8,192 grids and 16,384 n-body systems the same.  A batch of more
+    // warps than an SM holds blocks (32) keeps 128 threads: short calls then
+    // wait for blocks, 20,000 chains of 32 over 0.001 0.59 / 0.77 ms.
     bool any_block = false;
 };
+
+constexpr int kWarpBlocksPerSm = 32;  // the most blocks an SM holds
 
 // What the calling thread's last launch took (bode_last_launch).
 struct LaunchInfo {
@@ -59,9 +63,11 @@ struct is_double<double> {
 template <class Method, class Ctx>
 cudaError_t launch_method(const BatchArgs& a, const Ctx& ctx, const LaunchCfg& c) {
     constexpr int W = Method::W;
-    const int block = c.any_block && c.mapping == ODE_MAP_THREAD && is_double<typename Method::R>::value ? 32 : c.block;
-    const size_t smem = sizeof(float) * Method::SMEM_FLOATS * (size_t)block;
     const int64_t threads = a.nsys * W;
+    const bool warp_block = c.any_block && c.mapping == ODE_MAP_THREAD && is_double<typename Method::R>::value &&
+                            threads <= kWarpBlocksPerSm * 32 * (int64_t)c.sm_count;
+    const int block = warp_block ? 32 : c.block;
+    const size_t smem = sizeof(float) * Method::SMEM_FLOATS * (size_t)block;
     g_last_launch = LaunchInfo{a.index != nullptr, W, block, c.mapping};
     if (smem > 48 * 1024) {  // above the default dynamic shared-memory limit: opt in
         cudaError_t e = cudaFuncSetAttribute(k_static<Method, Ctx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -96,22 +102,34 @@ enum { kMethodRkck = 0, kMethodRkc = 1 };
 // with four systems in it as much as a warp with one.  So where the batch
 // fills the GPU a system takes as few lanes as hold it at four points each
 // (more points a lane spill), and where it does not, a whole warp, which
-// has the shortest step.  Time is taken as rounds of warps over the SMs'
-// four sub-partitions times a step's FP64 work, in units of one point's:
-// G points a lane plus kOwn + kSum npts for the system (from the FP64
-// instruction counts of an RKC step: 150 a point, 110 a system and two per
-// point in the norm).  Measured on 32 points: 8,192 systems 68.3 ms wide,
-// 52.5 narrow; 608 systems wide 6.3 ms, where a round of the narrow kernel
-// takes 15.4.
-inline int grid_team_f64(int npts, int64_t nsys, int sm_count) {
-    constexpr double kOwn = 0.75, kSum = 0.0133;
+// has the shortest step.  How much filling that takes depends on what a warp
+// loses to its longest system: little for grids by RKC, a third to a half of
+// the time for RKCK and for chains (whose mu spans more than a grid's
+// diffusion), unless the systems of a warp are alike (a batch read through an
+// order).  Measured, narrow / wide, by systems (608 sub-partitions):
+//   grids by RKC, 1-32 points   1,500: 0.97-1.28   2,500: 0.47-0.75   10,000: 0.18-0.66
+//     48, 64 points             1,000: 1.10        2,500: 0.91-1.03   10,000: 0.81
+//   grids by RKCK, <= 16        1,500: 0.94-1.59   2,500: 0.53-1.01   10,000: 0.15-0.66
+//     24-64, in order / not     5,000: 0.84-0.89 / 1.08-1.23
+//   chains by RKC, <= 16        2,500: 1.0-1.34    5,000: 0.70-0.88   10,000: 0.42-0.68
+//     24-64, in order / not     5,000: 0.80-0.87 / 1.06-1.12
+//   chains by RKCK, <= 8        5,000: 1.0-1.06    7,000: 0.79-0.87
+//     in order, 12-32 / 48, 64  5,000: 1.2 / 0.9   7,000: 0.98 / 0.8  10,000: 0.73-0.91 / 0.8
+inline int grid_team_f64(int npts, int64_t nsys, int sm_count, bool chain, int method, bool ordered) {
     int w = 1;
     while (w < 32 && 4 * w < npts) w *= 2;
-    const int64_t slots = 4 * (int64_t)sm_count;
-    auto rounds = [&](int lanes) { return (double)(((nsys * lanes + 31) / 32 + slots - 1) / slots); };
-    const double system = kOwn + kSum * npts;
-    const double narrow = rounds(w) * (4.0 + system), wide = rounds(32) * ((npts + 31) / 32 + system);
-    return narrow < wide ? w : 32;
+    const double wide = (double)nsys / (4 * sm_count), narrow = wide * w / 32;  // rounds of warps
+    const bool rkck = method == kMethodRkck;
+    bool take;
+    if (!chain && !rkck)
+        take = wide >= 4;
+    else if (ordered && narrow >= 2)
+        take = !(chain && rkck) || narrow >= 2.8 || wide >= 11;
+    else if (!chain)
+        take = w <= 4 && wide >= 4;
+    else
+        take = rkck ? w <= 2 && wide >= 11 : w <= 4 && wide >= 8;
+    return take ? w : 32;
 }
 
 // Per-family dispatch (defined in k_*.cu).  Each sets *ok = false when the
