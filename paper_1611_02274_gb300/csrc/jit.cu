@@ -399,7 +399,7 @@ struct JitKernels {
 };
 
 std::mutex g_jit_mu;
-std::map<std::string, JitKernels> g_cache;  // key: device + source hash + form
+std::map<std::string, JitKernels> g_cache;  // by cache_key
 
 // net: the two-float variant with the warp-level code (work queue, in-kernel
 // network); the other forms have one variant
@@ -550,10 +550,15 @@ int load_image(const JitImage& img, JitKernels* out, std::string* err) {
     return ODE_OK;
 }
 
+// What a form's kernels depend on.  The network stands for its source, which
+// is written from it alone (registration clears the entry, so unused slots and
+// padding are zero): every launch asks for its kernels, and writing the source
+// to hash it took the host 200 us of each (380 in two-float, whose call asks
+// twice), 230 and 440 with the packed form in it; the bytes take 1.
 std::string cache_key(const RhsEntry& r, int method, int prec, bool net, int dev) {
-    char key[128];
-    snprintf(key, sizeof(key), "%d/%d/%d/%d/%016llx/%d/%d", dev, method, prec, (int)net,
-             (unsigned long long)fnv1a(model_source(r)), jit_min_blocks(prec), jit_lockstep(prec));
+    const int32_t form[] = {dev, method, prec, (int32_t)net, jit_min_blocks(prec), jit_lockstep(prec), r.neq};
+    std::string key(reinterpret_cast<const char*>(form), sizeof(form));
+    key.append(reinterpret_cast<const char*>(&r.net), sizeof(r.net));
     return key;
 }
 
