@@ -52,8 +52,9 @@ struct RkcF2 {
     // Register budget of the warp-wide kernels (they wait on the latency of
     // the sums' chains, so warps count): one point a lane 128 instead of 141,
     // 32-point grids, 65,536 systems 30.8 -> 28.3 ms; four points 168
-    // instead of 234, the mixed batch of 32,768 systems 64.6 -> 57.8 ms.
-    static constexpr int kMaxRegs = W == 32 ? (P == 2 ? 128 : P >= 8 ? 168 : 255) : 255;
+    // instead of 234, the mixed batch of 32,768 systems 64.6 -> 57.8 ms; two
+    // points 168, three blocks of 128 threads an SM.
+    static constexpr int kMaxRegs = W == 32 ? (P == 2 ? 128 : 168) : 255;
     // the proposal network at the spectral-radius points (one thread per
     // system, up to 32 components + the parameter)
     using R = F2;
@@ -187,6 +188,18 @@ struct RkcF2 {
     // 168 registers, 1M systems in cost order 131.2 -> 118.7 ms (with the
     // packed arithmetic).
     static constexpr bool kUniform = W == 1;
+    // Small states keep a stage's coefficients in registers, asked for at the
+    // end of the stage before: without pressure on the registers a read where
+    // they are used only adds its latency to every stage (van der Pol RKC,
+    // 12,000 systems 5.04 / 5.22 ms, 8,000 chains of 64 oscillators 3.72 /
+    // 5.03).
+    static constexpr bool kEarlyCoef = P <= 4 && kMaxRegs > 128;
+    struct HeldCoef {
+        CoefSource cs;
+        float4 hi, lo;
+    };
+    struct NoCoef {};
+    typename Pick<kEarlyCoef, HeldCoef, NoCoef>::type held;
     __device__ HT hmax(const BatchArgs& a) const { return kUniform ? pick_ht(a.u.hmax, a.u.hmaxf) : hmax_; }
     __device__ HT hmin(const BatchArgs& a) const { return kUniform ? pick_ht(a.u.hmin, a.u.hminf) : hmin_; }
     __device__ float rtolf(const BatchArgs& a) const { return kUniform ? a.u.rtolf : rtolf_; }
@@ -592,6 +605,10 @@ struct RkcF2 {
 #pragma unroll(P <= 64 ? P : 4)
         for (int q = 0; q < NP; ++q) d1[q] = mul_lazy(mut1h, Fn[q]);  // a product: its pair stays near-normal
         j = 2;
+        if constexpr (kEarlyCoef) {
+            held.cs = cs;
+            cs.stagef2(2, held.hi, held.lo);
+        }
         phase = PH_STAGE;
     }
 
@@ -608,8 +625,14 @@ struct RkcF2 {
     __device__ void stage_consume(const BatchArgs& a, const F2* f) {
         float4 chi, clo;  // (mu_j, nu_j, mu~_j, gamma~_j), leading / trailing words
         CoefSource cs;
-        cs.start(m, a);
-        cs.stagef2(j, chi, clo);
+        if constexpr (kEarlyCoef) {
+            cs = held.cs;
+            chi = held.hi;
+            clo = held.lo;
+        } else {
+            cs.start(m, a);
+            cs.stagef2(j, chi, clo);
+        }
         const F2 mu(chi.x, clo.x);
         const F2x2 muth(F2(chi.z, clo.z) * hh);
         const bool keep = j < m;  // d_{j-1} is the next stage's d_{j-2}
@@ -633,7 +656,10 @@ struct RkcF2 {
             }
         }
         j += 1;
-        if (j > m) phase = PH_FINAL;
+        if (j > m)
+            phase = PH_FINAL;
+        else if constexpr (kEarlyCoef)
+            held.cs.stagef2(j, held.hi, held.lo);
     }
 
     __device__ static constexpr int i_second(int q) { return q + NP; }
