@@ -73,8 +73,14 @@ struct RkcF2 {
     // d_{j-2}, needed only from the third stage on: for one-thread systems a
     // row of packs in shared memory (an odd number of 16-byte packs per row:
     // no bank conflicts), so a two-stage step -- the common case at tight
-    // tolerances -- touches it never and holds no registers for it
-    static constexpr int D2_SMEM = (W == 1 && P <= 32) ? 4 * (NP | 1) : 0;
+    // tolerances -- touches it never and holds no registers for it.
+    // A state of three slots or fewer fits in registers with all it needs;
+    // rows and kernel arguments (kUniform) only add their latency there: van
+    // der Pol RKC, 12,000 systems 4.50 / 5.01 ms.  Without a row there is no
+    // in-kernel network and no joined estimate, which change results in the
+    // work queue: they are for four components and more.
+    static constexpr bool kSmall = W == 1 && P <= 3;
+    static constexpr int D2_SMEM = (W == 1 && !kSmall && P <= 32) ? 4 * (NP | 1) : 0;
     // the state y_n, read at the evaluation points, the error weights and
     // the accept only: for one-thread systems a shared-memory row too, so
     // that no state pair stays live across the right-hand-side evaluation
@@ -84,7 +90,8 @@ struct RkcF2 {
     // system with rows in shared memory: up to 32 components + the
     // parameter, the BF16 features staged in the d_{j-2} row)
     static constexpr int kMlpKs = (P + 1 + 15) / 16;
-    static constexpr bool kWarpPropose = NET && W == 1 && P <= 32 && D2_SMEM >= 8 * kMlpKs && Y_SMEM > 0;
+    static constexpr bool kWarpPropose = NET && W == 1 && P >= 4 && P <= 32;
+    static_assert(!kWarpPropose || (D2_SMEM >= 8 * kMlpKs && Y_SMEM > 0), "room for the features");
     static constexpr int kJoin = 12;  // steps before its point a system joins a warp's network evaluation
     mutable F2 vreg[V_SMEM ? 1 : P];
     mutable F2x2 d2reg[D2_SMEM ? 1 : NP];
@@ -180,14 +187,14 @@ struct RkcF2 {
     float rtolf_, atolf_, c3_old, dynrm, sig;
     int32_t n_acc, n_rej, n_rhs, n_sr, status, mmax_, num_step, sr_step, n_;
     // One-thread systems come in uniform batches (ragged plans give a system
-    // a team), so the interval's and tolerances' scalars are kernel
+    // a team), so for larger states the interval's and tolerances' scalars are kernel
     // arguments, read where a step needs them (the host converts them once);
     // stage coefficients are read from the table where they are used.  What
     // stays in registers across the right-hand-side evaluation decides what
     // the compiler spills: 472 -> 120 bytes in the 13-species kernel at its
     // 168 registers, 1M systems in cost order 131.2 -> 118.7 ms (with the
     // packed arithmetic).
-    static constexpr bool kUniform = W == 1;
+    static constexpr bool kUniform = W == 1 && !kSmall;
     // Small states keep a stage's coefficients in registers, asked for at the
     // end of the stage before: without pressure on the registers a read where
     // they are used only adds its latency to every stage (van der Pol RKC,
