@@ -175,7 +175,10 @@ int validate_desc(const ode_rhs_desc* d, RhsEntry* r) {
         dv.insert(dv.end(), d->beta, d->beta + R);
         dv.insert(dv.end(), d->Ea, d->Ea + R);
         for (int j = 0; j < R; ++j) dv.push_back(2.302585092994046 * d->log10A[j]);
-        for (int i = 0; i < S; ++i) dv.push_back(1.0 / d->mol_weights[i]);
+        for (int i = 0; i < S; ++i) {  // as xm::reciprocal gives it
+            const double w = d->mol_weights[i];
+            dv.push_back(w >= std::ldexp(1.0, -100) && w <= std::ldexp(1.0, 100) ? 1.0 / w : 0.0);
+        }
         for (int i = 0; i < S; ++i) dv.push_back(8.314462618 / d->mol_weights[i]);
         if (dv.size() % 2) dv.push_back(0.0);  // the float4 section starts 16-byte aligned
         std::vector<float> fv;

@@ -70,32 +70,23 @@ __device__ __forceinline__ double small_int(int k) { return (double)(float)k; }
 // a / b with r = 1 / b correctly rounded and b in [2^-100, 2^100]: one
 // residual correction of a r rounds correctly (Markstein, IBM J. Res. Dev.
 // 34 (1990) 111: with a correctly rounded reciprocal and a quotient within
-// one ulp, fma(residual, r, q) is the rounded quotient).  Three FP64
-// instructions instead of a division's eight.  Dividends outside
+// one ulp, q - (q b - a) r with fused operations is the rounded quotient).
+// Three FP64 instructions instead of a division's eight.  Dividends outside
 // [2^-700, 2^700], where the residual could round, divide as usual; zeros
-// take the short way.  Pass r = 0 for a divisor outside the range.
+// take the short way and keep their sign.  Pass r = 0 for a divisor outside
+// the range; one that is not positive divides as usual too.
 static __device__ __noinline__ double div_general(double a, double b) { return a / b; }
 __device__ __forceinline__ double div_by(double a, double b, double r) {
     const unsigned hi = (unsigned)__double2hiint(a) & 0x7fffffffu;
     const bool ordinary = hi - (323u << 20) <= (1400u << 20) || (hi | (unsigned)__double2loint(a)) == 0u;
-    if (!ordinary || __double2hiint(r) == 0) return div_general(a, b);
+    if (!ordinary || __double2hiint(r) <= 0) return div_general(a, b);
     const double q = a * r;
-    return fma(fma(-q, b, a), r, q);
+    return fma(-fma(q, b, -a), r, q);
 }
-// The reciprocal div_by takes.  From the hardware's first approximation
-// (about 20 bits) one third-order step, y (1 + e + e^2) with e = 1 - b y,
-// leaves it within an ulp, and one residual correction rounds it correctly
-// for every significand but the one of all ones (Markstein), which divides:
-// five FP64 instructions instead of a division's eight.
+// The reciprocal div_by takes: CUDA's own, 0 for a divisor outside the range.
 __device__ __forceinline__ double reciprocal(double b) {
-    const unsigned hi = (unsigned)__double2hiint(b) & 0x7fffffffu;
-    if (!(hi - (923u << 20) <= (200u << 20))) return 0.0;
-    if ((hi & 0xfffffu) == 0xfffffu) return div_general(1.0, b);
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    double e = fma(-b, y, 1.0);
-    y = fma(fma(e, e, e), y, y);
-    return fma(fma(-b, y, 1.0), y, y);
+    const unsigned hi = (unsigned)__double2hiint(b);
+    return hi - (923u << 20) <= (200u << 20) ? __drcp_rn(b) : 0.0;
 }
 
 // 1/(2i+1) for i = 11 .. 0, Horner in t^2; log x from f and its exponent
