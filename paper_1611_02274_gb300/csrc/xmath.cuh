@@ -85,8 +85,8 @@ __device__ __forceinline__ double div_by(double a, double b, double r) {
 }
 // The reciprocal div_by takes: CUDA's own, 0 for a divisor outside the range.
 __device__ __forceinline__ double reciprocal(double b) {
-    const unsigned hi = (unsigned)__double2hiint(b);
-    return hi - (923u << 20) <= (200u << 20) ? __drcp_rn(b) : 0.0;
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(b);
+    return bits - (923ull << 52) <= (200ull << 52) ? __drcp_rn(b) : 0.0;
 }
 
 // 1/(2i+1) for i = 11 .. 0, Horner in t^2; log x from f and its exponent
