@@ -114,7 +114,9 @@ extern "C" {
                                 the choice is cached per rhs / method / precision / device.
                                 Smaller batches, and calls on a capturing stream, use
                                 ODE_MAP_THREAD with 128-thread blocks (32-thread blocks in
-                                plain FP64 up to 32 warps per SM).  Ragged plans: see
+                                plain FP64 up to 32 warps per SM); forms other
+                                than plain FP64 take a cached choice for smaller
+                                batches too.  Ragged plans: see
                                 ode_ragged_plan_create */
 #define ODE_MAP_THREAD 1     /* one thread per system, one launch over the batch (the paper's) */
 #define ODE_MAP_QUEUE 2      /* persistent kernel, one thread per system, systems pulled from a

@@ -519,7 +519,12 @@ int tune_mapping(Workspace* ws, int32_t handle, const RhsEntry& rhs, int meth, i
     cudaGetDevice(&dev);
     const auto key = std::make_tuple(handle, meth, prec, (int)use_jit, dev, block_req);
     auto it = g_map_tuned.find(key);
-    if (it != g_map_tuned.end()) {
+    // Plain FP64: a choice timed on a batch that fills the device says nothing
+    // about one that does not (100 van der Pol systems: a lane pair each in
+    // one-warp blocks, whatever a large batch before them took).  The other
+    // forms' default is not made for a size, and the timed block is as good or
+    // better (20,000-30,000 two-float networks 64 / 128 threads 5.32 / 5.70 ms).
+    if ((a.nsys >= kTuneMinSystems || prec != ODE_PREC_FP64) && it != g_map_tuned.end()) {
         cfg->mapping = it->second.first;
         cfg->block = it->second.second;
         cfg->any_block = false;
