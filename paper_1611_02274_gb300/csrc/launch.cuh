@@ -43,6 +43,7 @@ struct LaunchCfg {
 };
 
 constexpr int kWarpBlocksPerSm = 32;  // the most blocks an SM holds
+constexpr size_t kSmemPerBlock = 227 * 1024;
 
 // What the calling thread's last launch took (bode_last_launch).
 struct LaunchInfo {
@@ -69,10 +70,15 @@ cudaError_t launch_method(const BatchArgs& a, const Ctx& ctx, const LaunchCfg& c
     const int block = warp_block ? 32 : c.block;
     const size_t smem = sizeof(float) * Method::SMEM_FLOATS * (size_t)block;
     g_last_launch = LaunchInfo{a.index != nullptr, W, block, c.mapping};
-    if (smem > 48 * 1024) {  // above the default dynamic shared-memory limit: opt in
-        cudaError_t e = cudaFuncSetAttribute(k_static<Method, Ctx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024) {
+        // Above the default dynamic shared-memory limit: opt in, always to what
+        // the largest block takes (the attribute is the kernel's, and another
+        // entry point's thread may launch it with a smaller block in between).
+        constexpr size_t kMost = sizeof(float) * Method::SMEM_FLOATS * BODE_MAX_THREADS;
+        const size_t limit = smem > kSmemPerBlock ? smem : kMost < kSmemPerBlock ? kMost : kSmemPerBlock;
+        cudaError_t e = cudaFuncSetAttribute(k_static<Method, Ctx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_queue<Method, Ctx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = cudaFuncSetAttribute(k_queue<Method, Ctx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
         if (e != cudaSuccess) return e;
     }
     if (c.mapping == ODE_MAP_QUEUE) {
