@@ -156,7 +156,8 @@ struct UniformScalars {
         hminf = (float)hmin;
         rtolf = (float)rtol;
         atolf = (float)atol;
-        mmax = (int)round(sqrt(rtol / (10.0 * kUround)));
+        // clamped before it is converted, which a host need not do as the device does
+        mmax = (int)fmin(round(sqrt(rtol / (10.0 * kUround))), 2147483647.0);
         if (mmax < 2) mmax = 2;
     }
 };
