@@ -16,6 +16,9 @@ kinetics families.
 
 For N > 1 run under torch.distributed.run: every rank integrates its own
 batch (seed = rank), no collective on the data path (weak scaling).
+
+Prints one JSON line of the main leg with a rate per form and leg; the whole
+record goes to bench_detail.json (--detail).
 """
 from __future__ import annotations
 
@@ -526,7 +529,10 @@ def run_ours(args):
         if rank == 0:
             out["global_steps"] = split
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as fh:
+                json.dump(out, fh, indent=1)
+        print(short_line(out), flush=True)
     B.release(h)
     if net is not None:
         net.release()
@@ -1201,6 +1207,44 @@ def c1_leg(args, B, torch, dev, stream, rank, world, barrier):
     return res
 
 
+# What the printed line keeps of the roofline, each form and each leg; the
+# whole record goes to the file of --detail.
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "status_ok_frac",
+             "rhs_evals_per_s", "cpu_baseline", "speedup_chosen_vs_plain", "fp64_fma_measured_tflops",
+             "fp32_fma_measured_tflops")
+LINE_ROOFLINE = ("bound", "achieved", "peak", "unit", "frac", "frac_of_measured", "traffic", "kernel", "kernel_ms",
+                 "prepass_ms")
+LINE_RATES = {  # leg: (path to its rate, ...)
+    "c0_vdp_rkck": ("nsys_1048576.two_float.systems_per_s", "nsys_1048576.systems_per_s"),
+    "c1_bruss_rkc": ("f2_lean.systems_per_s", "plain_fp64.systems_per_s"),
+    "pleiades_rkck": ("systems_per_s",),
+}
+
+
+def short_line(out: dict) -> str:
+    """The record as one line of a few kB: required keys, the roofline, a rate and an error per form, rates of legs."""
+    line = {k: out[k] for k in LINE_KEYS if k in out}
+    if "roofline" in out:
+        line["roofline"] = {k: out["roofline"].get(k) for k in LINE_ROOFLINE}
+    if "forms" in out:
+        line["forms"] = {n: {"value": f["value"], "p999_err": f.get("err_vs_fp64_oracle_p999")}
+                         for n, f in out["forms"].items()}
+    if "target" in out:
+        line["chosen_meets_target"] = out["target"]["chosen_meets"]
+    legs = {}
+    for leg, paths in LINE_RATES.items():
+        for path in paths:
+            v = out.get(leg)
+            for key in path.split("."):
+                v = v.get(key) if isinstance(v, dict) else None
+            if isinstance(v, float):
+                legs[f"{leg}.{path.removesuffix('.systems_per_s')}"] = v
+    if legs:
+        line["legs"] = legs
+    return json.dumps(line)
+
+
 def err_stats(y, ref_y, atol, rtol):
     """Per-system final-state error against the oracle: max_i |y - y_ref| /
     (|y_ref| + atol), summarised over the systems, and in tolerance units."""
@@ -1334,6 +1378,8 @@ def main():
     ap.add_argument("--pleiades-steps", type=int, default=3)
     ap.add_argument("--split-steps", type=int, default=10, help="global steps of the outer-loop leg (0 skips it)")
     ap.add_argument("--split-reps", type=int, default=2)
+    ap.add_argument("--detail", default=os.path.join(ROOT, "bench_detail.json"),
+                    help="file for the whole record (every leg and form); empty: none")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)   # at least three untimed warm-up steps
     if args.impl == "reference":
