@@ -114,7 +114,7 @@ extern "C" {
                                 the choice is cached per rhs / method / precision / device.
                                 Smaller batches, and calls on a capturing stream, use
                                 ODE_MAP_THREAD with 128-thread blocks (32-thread blocks in
-                                plain FP64 up to 32 warps per SM); forms other
+                                plain FP64); forms other
                                 than plain FP64 take a cached choice for smaller
                                 batches too.  Ragged plans: see
                                 ode_ragged_plan_create */

@@ -205,7 +205,7 @@ std::string packed_rhs(const MassActionNet& net) {
 }
 
 // The network as a Model (see rhs.cuh for the interface): rate constants in
-// registers, f written as straight-line code whose per-species accumulation
+// registers (FP32 forms) or a shared-memory row, f written as straight-line code whose per-species accumulation
 // order is the reaction order (reactants, then products).
 std::string model_source(const RhsEntry& r) {
     const MassActionNet& net = r.net;
@@ -215,7 +215,7 @@ std::string model_source(const RhsEntry& r) {
       << "  static constexpr int W = 1, PER = " << S << ";\n"
       << "  using Ctx = bode::NoCtx;\n"
       << "  template <class R> struct Sys {\n"
-      << "    bode::ConstStore<R, " << NR << "> k;  // registers, or a shared-memory row (two-float forms)\n"
+      << "    bode::ConstStore<R, " << NR << "> k;  // registers, or a shared-memory row (plain and two-float forms)\n"
       << "    static constexpr int CONST_SMEM = bode::ConstStore<R, " << NR << ">::SMEM_FLOATS;\n"
       << "    __device__ void bind_consts(float* row) { k.bind(row); }\n"
       << "    int n;\n"
@@ -727,9 +727,7 @@ int jit_launch(const RhsEntry& r, int method, int prec, const BatchArgs& a, cons
     NoCtx ctx;
     BatchArgs args = a;
     void* params[] = {&args, &ctx};
-    const bool warp_block = c.any_block && c.mapping == ODE_MAP_THREAD && prec == ODE_PREC_FP64 &&
-                            a.nsys <= kWarpBlocksPerSm * 32 * (int64_t)c.sm_count;  // as in launch_method
-    const int block = warp_block ? 32
+    const int block = c.any_block && c.mapping == ODE_MAP_THREAD && prec == ODE_PREC_FP64 ? 32  // as in launch_method
                       : c.block > jit_max_block(prec) ? jit_max_block(prec) : c.block;
     // the generated model is one thread per system with PER = species count
     const size_t smem = sizeof(float) * (size_t)k.smem_floats * (size_t)block;

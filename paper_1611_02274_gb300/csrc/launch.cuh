@@ -36,13 +36,11 @@ struct LaunchCfg {
     // blocks leave a batch of a few warps per SM unevenly spread.  Measured,
     // 128 / 32 threads: kinetics, 1,000 systems 94.9 / 83.2 ms; 32-point
     // grids, 2,500 systems 26.0 / 18.6; van der Pol, 30,000 systems 7.04 /
-    // 6.11; 8,192 grids and 16,384 n-body systems the same.  A batch of more
-    // warps than an SM holds blocks (32) keeps 128 threads: short calls then
-    // wait for blocks, 20,000 chains of 32 over 0.001 0.59 / 0.77 ms.
+    // 6.11; 8,192 grids and 16,384 n-body systems the same; kinetics, 5,000
+    // systems of 12 species (more warps than an SM holds blocks) 115.7 / 106.1.
     bool any_block = false;
 };
 
-constexpr int kWarpBlocksPerSm = 32;  // the most blocks an SM holds
 constexpr size_t kSmemPerBlock = 227 * 1024;
 
 // What the calling thread's last launch took (bode_last_launch).
@@ -65,9 +63,7 @@ template <class Method, class Ctx>
 cudaError_t launch_method(const BatchArgs& a, const Ctx& ctx, const LaunchCfg& c) {
     constexpr int W = Method::W;
     const int64_t threads = a.nsys * W;
-    const bool warp_block = c.any_block && c.mapping == ODE_MAP_THREAD && is_double<typename Method::R>::value &&
-                            threads <= kWarpBlocksPerSm * 32 * (int64_t)c.sm_count;
-    const int block = warp_block ? 32 : c.block;
+    const int block = c.any_block && c.mapping == ODE_MAP_THREAD && is_double<typename Method::R>::value ? 32 : c.block;
     const size_t smem = sizeof(float) * Method::SMEM_FLOATS * (size_t)block;
     g_last_launch = LaunchInfo{a.index != nullptr, W, block, c.mapping};
     if (smem > 48 * 1024) {
