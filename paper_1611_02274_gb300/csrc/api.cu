@@ -171,7 +171,6 @@ int validate_desc(const ode_rhs_desc* d, RhsEntry* r) {
         std::vector<double> dv;
         dv.insert(dv.end(), d->mol_weights, d->mol_weights + S);
         dv.insert(dv.end(), d->thermo, d->thermo + 4 * S);
-        dv.insert(dv.end(), d->log10A, d->log10A + R);
         dv.insert(dv.end(), d->beta, d->beta + R);
         dv.insert(dv.end(), d->Ea, d->Ea + R);
         for (int j = 0; j < R; ++j) dv.push_back(2.302585092994046 * d->log10A[j]);
@@ -243,8 +242,7 @@ int validate_desc(const ode_rhs_desc* d, RhsEntry* r) {
         kd.kmax = d->kmax;
         kd.W = dp;
         kd.thermo = dp + S;
-        kd.log10A = dp + 5 * S;
-        kd.beta = kd.log10A + R;
+        kd.beta = dp + 5 * S;
         kd.Ea = kd.beta + R;
         kd.ln10A = kd.Ea + R;
         kd.rW = kd.ln10A + R;
@@ -380,7 +378,8 @@ void default_mapping(LaunchCfg* cfg, int block_req) {
 //                               below the line        above it
 //   van der Pol RKCK, FP64      20,000 over 0.3 1.02  20,000 over 1 0.90, 250,000 over 0.1 0.56
 //     two-float (FP32 1.2-2.9)  60,000 over 0.1 1.64  60,000 over 10 0.77, 250,000 over 1 0.47
-//   RKC, FP64 (grids, chains)   20,000 over 3 1.05    60,000 over 0.01 0.89, over 1 0.59
+//     chains                    20,000 of 4 over 0.01 1.27  over 0.5 0.87, over 4 0.82
+//   RKC, FP64                   20,000 over 3 1.05    over 20 0.94, 60,000 over 0.01 0.89
 //     two-float                 60,000 over 0.3 1.09  250,000 over 0.01 0.89, over 1 0.52
 //   networks (kmax 1e6), FP64   60,000 over 1e-6 0.99 over 1e-5 0.76
 //     two-float                 over 1e-8 1.04        over 1e-5 0.88
@@ -392,8 +391,8 @@ int auto_order(const RhsEntry& rhs, int meth, int prec, const BatchArgs& a, int 
     if (a.carry != nullptr || a.mlp != nullptr || a.nsys > INT32_MAX) return -1;
     const bool f64 = prec == ODE_PREC_FP64, rkc = meth == kMethodRkc;
     int lanes = 32;
-    double units = a.tend - a.t0, rounds_min = rkc || rhs.kind != ODE_RHS_VDP ? 2.0 : 1.0;
-    double work_min = rkc ? 0.03 : 0.9;  // rounds x units
+    double units = a.tend - a.t0, rounds_min = rkc || rhs.kind == ODE_RHS_BRUSS1D ? 2.0 : 1.0;
+    double work_min = rkc ? 0.03 : rhs.kind == ODE_RHS_VDP_CHAIN ? 0.5 : 0.9;  // rounds x units
     if (!f64) rounds_min = rkc ? 5.0 : 3.0, work_min = rkc ? 0.1 : 10.0;
     switch (rhs.kind) {
     case ODE_RHS_VDP: lanes = 1; break;
@@ -411,6 +410,7 @@ int auto_order(const RhsEntry& rhs, int meth, int prec, const BatchArgs& a, int 
         break;
     }
     const double rounds = (double)(a.nsys * lanes) / (32 * 4 * (double)sm_count);
+    if (rkc && units >= 10.0) rounds_min = 1.0;
     return lanes < 32 && rounds > rounds_min && rounds * units >= work_min ? (int)kCostParam : -1;
 }
 // whether a launch may take the systems in another order
