@@ -104,8 +104,7 @@ struct KinDevice {
     double kmin, kmax;
     const double* W;        // [S]
     const double* thermo;   // [S][4]
-    const double* log10A;   // [R]
-    const double* beta;
+    const double* beta;     // [R]
     const double* Ea;
     // the plain form's constants of the mechanism, each the correctly
     // rounded value its expression would take in every evaluation
