@@ -483,7 +483,12 @@ struct OrderScratch {
                 cudaGetLastError();  // not the caller's error: the batch keeps its order
             }
         }
-        if (!fit && oldest && cudaStreamWaitEvent(s, oldest->done, 0) == cudaSuccess) fit = oldest;
+        if (!fit && oldest) {
+            if (cudaStreamWaitEvent(s, oldest->done, 0) == cudaSuccess)
+                fit = oldest;
+            else
+                cudaGetLastError();
+        }
         if (!fit) return false;
         buf = fit;
         buf->turn = ++ws->auto_turn;
